@@ -6,6 +6,7 @@
 // f16x2, never contracted), subnormals kept.  Global traffic is 128-bit.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cstring>
 
 #include "../../include/pf16.h"
@@ -1422,13 +1423,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-unsigned grid_for(long long work, int per_block, int cap) {
-  long long b = (work + per_block - 1) / per_block;
-  if (b < 1) b = 1;
-  if (b > cap) b = cap;
-  return (unsigned)b;
-}
-
 }  // namespace
 
 static BnPlan bn_stat_plan(long long chunks, int ctas_per_sm) {
@@ -2021,34 +2015,82 @@ cudaError_t launch_bn_relu_pool_fwd(const BnLaunch& b, const uint8_t* conv_stats
 
 // ============================================================================
 // Global average pooling (halving tree over hw padded to 2^L, x rn(2^L/hw)).
+// Bound by HBM: x is read once forward, written once backward.
+//
+// Forward: a CTA takes 32 channel groups of 8 (a warp reads 512 consecutive
+// bytes of a pixel); its warps share the padded pixels in aligned runs of
+// 2^L / 8 (at least 8), each summed as perfect subtrees of 8 with all eight
+// loads in flight, and the runs' nodes meet in shared memory -- the same
+// perfect tree as a pixel-by-pixel counter, whose one load in flight per
+// thread made 256 x 49 x 2048 take 37.5 us (1.4 TB/s); now 17 us.
+// Backward: a thread scales its channel group once and writes it to every
+// eighth pixel (15.3 -> 12.2 us at that size).
 // ============================================================================
-__global__ void k_avgpool_fwd(const uint16_t* __restrict__ x, uint16_t* __restrict__ y, int N, int HW,
-                              int C, int levels, uint16_t ratio) {
+constexpr int kPoolWarps = 8;
+
+__global__ void __launch_bounds__(32 * kPoolWarps)
+    k_avgpool_fwd(const uint16_t* __restrict__ x, uint16_t* __restrict__ y, int N, int HW, int C, int levels,
+                  uint16_t ratio) {
   pdl_wait();
-  const int tc = C / 8;
+  __shared__ uint4 node[kPoolWarps][32];
+  const int tc = C / 8, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long total = (long long)N * tc;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int cg = (int)(t % tc);
-    const long long n = t / tc;
-    Tree4<12, true> tree;
-    for (int i = 0; i < HW; ++i)
-      tree.push(__ldg(reinterpret_cast<const uint4*>(x + (n * HW + i) * C) + cg));
-    reinterpret_cast<uint4*>(y)[t] = mul4(tree.finish(levels), dup2(ratio));
+  const long long t = (long long)blockIdx.x * 32 + lane;
+  // warps in use and pixels per warp (powers of two; run * warps = 2^levels)
+  const int warps = levels <= 3 ? 1 : (levels >= 6 ? kPoolWarps : 1 << (levels - 3));
+  const int run = (1 << levels) / warps;
+  const int nb = run < 8 ? run : 8;  // leaves per batch
+  if (w < warps) {
+    const int cg = t < total ? (int)(t % tc) : 0;
+    const long long n = t < total ? t / tc : 0;
+    const uint4* src = reinterpret_cast<const uint4*>(x) + n * HW * tc + cg;
+    uint4 acc = zero4();
+    Tree4<12, true> tree;  // over the run's batches, when it has several
+    for (int i0 = 0; i0 < run; i0 += 8) {
+      uint4 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int px = w * run + i0 + i;
+        v[i] = (t < total && i < nb && px < HW) ? __ldg(src + (long long)px * tc) : zero4();
+      }
+#pragma unroll
+      for (int h = 1; h < 8; h *= 2)
+#pragma unroll
+        for (int i = 0; i < 8; i += 2 * h)
+          if (i + h < nb) v[i] = hmerge4(v[i], v[i + h]);
+      if (run <= 8) {
+        acc = v[0];
+        break;
+      }
+      tree.push(v[0]);
+    }
+    if (run > 8) acc = tree.finish(ceil_log2(run / 8));
+    node[w][lane] = acc;
   }
+  __syncthreads();
+  if (w != 0 || t >= total) return;
+  uint4 v[kPoolWarps];
+#pragma unroll
+  for (int i = 0; i < kPoolWarps; ++i) v[i] = i < warps ? node[i][lane] : zero4();
+#pragma unroll
+  for (int h = 1; h < kPoolWarps; h *= 2)
+#pragma unroll
+    for (int i = 0; i < kPoolWarps; i += 2 * h)
+      if (i + h < warps) v[i] = hmerge4(v[i], v[i + h]);
+  reinterpret_cast<uint4*>(y)[t] = mul4(v[0], dup2(ratio));
 }
 
-__global__ void k_avgpool_bwd(const uint16_t* __restrict__ dy, uint16_t* __restrict__ dx, int N,
-                              int HW, int C, uint16_t inv) {
+__global__ void __launch_bounds__(32 * kPoolWarps)
+    k_avgpool_bwd(const uint16_t* __restrict__ dy, uint16_t* __restrict__ dx, int N, int HW, int C, uint16_t inv) {
   pdl_wait();
-  const int tc = C / 8;
-  const long long total = (long long)N * HW * tc;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int cg = (int)(t % tc);
-    const long long n = t / ((long long)HW * tc);
-    reinterpret_cast<uint4*>(dx)[t] = mul4(__ldg(reinterpret_cast<const uint4*>(dy + n * C) + cg), dup2(inv));
-  }
+  const int tc = C / 8, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long t = (long long)blockIdx.x * 32 + lane;
+  if (t >= (long long)N * tc) return;
+  const long long n = t / tc;
+  const int cg = (int)(t - n * tc);
+  const uint4 v = mul4(__ldg(reinterpret_cast<const uint4*>(dy) + t), dup2(inv));
+  uint4* dst = reinterpret_cast<uint4*>(dx) + n * HW * tc + cg;
+  for (long long px = blockIdx.y * kPoolWarps + w; px < HW; px += gridDim.y * kPoolWarps) dst[px * tc] = v;
 }
 
 cudaError_t launch_avgpool_fwd(const uint16_t* x, uint16_t* y, int N, int HW, int C,
@@ -2057,15 +2099,19 @@ cudaError_t launch_avgpool_fwd(const uint16_t* x, uint16_t* y, int N, int HW, in
   while ((1 << L) < HW) ++L;
   const uint16_t ratio = f16_bits_host((float)((double)(1 << L) / HW));
   const long long total = (long long)N * (C / 8);
-  launch_pdl(k_avgpool_fwd, dim3(grid_for(total, 128, 152 * 16)), dim3(128), 0, s, x, y, N, HW, C, L, ratio);
+  launch_pdl(k_avgpool_fwd, dim3((unsigned)((total + 31) / 32)), dim3(32 * kPoolWarps), 0, s, x, y, N, HW, C, L, ratio);
   return counted_launches(1);
 }
 
 cudaError_t launch_avgpool_bwd(const uint16_t* dy, uint16_t* dx, int N, int HW, int C,
                                cudaStream_t s) {
   const uint16_t inv = f16_bits_host((float)(1.0 / HW));
-  const long long total = (long long)N * HW * (C / 8);
-  launch_pdl(k_avgpool_bwd, dim3(grid_for(total, 256, 152 * 16)), dim3(256), 0, s, dy, dx, N, HW, C, inv);
+  const long long total = (long long)N * (C / 8);
+  // the pixels of an image are shared by gridDim.y CTAs where the channel groups
+  // alone leave SMs idle (16 CTAs per SM wanted)
+  const long long gx = (total + 31) / 32;
+  const long long gy = std::max(1ll, std::min((HW + kPoolWarps - 1ll) / kPoolWarps, kGb300Sms * 16 / gx));
+  launch_pdl(k_avgpool_bwd, dim3((unsigned)gx, (unsigned)gy), dim3(32 * kPoolWarps), 0, s, dy, dx, N, HW, C, inv);
   return counted_launches(1);
 }
 
@@ -2074,9 +2120,16 @@ cudaError_t launch_avgpool_bwd(const uint16_t* dy, uint16_t* dx, int N, int HW, 
 // S = pairwise FP16 sum of exp(rn(l - m)), lse = rn(m + log S),
 // dlogits = rn(rn(exp(rn(l - lse)) - onehot) * rn(1/B)), loss_b = rn(lse - l_label);
 // then the batch mean of loss_b (halving tree) and dbias = pairwise column sums.
+// Both launches are bound by latency (256 x 1000 logits are half a megabyte):
+// a row's values stay in registers between its passes, and the columns' and
+// the losses' trees run over the rows in parallel.  (One thread per column
+// walking the rows, one thread for the losses: 59.3 us for the call at 256 x
+// 1000; now 12.2 us.)
 // ============================================================================
 namespace {
 constexpr int kSmThreads = 256;
+constexpr int kSmMaxPer = 4096 / kSmThreads;  // logits of a row per thread, at most
+constexpr int kColSegs = 32;                  // row segments of a column tree: one per warp
 
 __device__ __forceinline__ __half hb(uint16_t u) { return __ushort_as_half(u); }
 __device__ __forceinline__ uint16_t bh(__half h) { return __half_as_ushort(h); }
@@ -2090,35 +2143,38 @@ __global__ void __launch_bounds__(kSmThreads)
                    const int32_t* __restrict__ labels, int K, uint16_t invB,
                    uint16_t* __restrict__ dlogits, uint16_t* __restrict__ row_loss) {
   pdl_wait();
-  __shared__ float smax[kSmThreads / 32];
+  constexpr int kWarps = kSmThreads / 32;
+  __shared__ float smax[kWarps];
   __shared__ uint16_t ssum[kSmThreads];
-  __shared__ __half s_lse;
   const int b = blockIdx.x, t = threadIdx.x;
   const uint16_t* z = logits + (long long)b * K;
-  // pass 1: max of l
+  const int lab = labels[b];
+  // l = rn(z + bias) of the thread's columns t, t + 256, ...; their maximum
+  __half l[kSmMaxPer];
   float mx = -INFINITY;
-  for (int k = t; k < K; k += kSmThreads) {
-    const __half l = bias ? hadd(hb(z[k]), hb(bias[k])) : hb(z[k]);
-    mx = fmaxf(mx, __half2float(l));
+#pragma unroll
+  for (int i = 0; i < kSmMaxPer; ++i) {
+    const int k = t + i * kSmThreads;
+    if (k < K) {
+      l[i] = bias ? hadd(hb(z[k]), hb(bias[k])) : hb(z[k]);
+      mx = fmaxf(mx, __half2float(l[i]));
+    }
   }
 #pragma unroll
   for (int o = 16; o >= 1; o /= 2) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((t & 31) == 0) smax[t >> 5] = mx;
   __syncthreads();
-  if (t < 32) {
-    float v = t < kSmThreads / 32 ? smax[t] : -INFINITY;
 #pragma unroll
-    for (int o = 16; o >= 1; o /= 2) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (t == 0) smax[0] = v;
-  }
-  __syncthreads();
-  const __half m = __float2half_rn(smax[0]);  // exact: the max of binary16 values
-  // pass 2: S = sum exp(rn(l - m)) as a pairwise tree (thread trees, then across threads)
+  for (int w = 0; w < kWarps; ++w) mx = fmaxf(mx, smax[w]);
+  const __half m = __float2half_rn(mx);  // exact: the max of binary16 values
+  // S = sum exp(rn(l - m)) as a pairwise tree: the thread's columns (binary
+  // counter), then threads t and t + 128, t + 64, ..., t + 1
   uint16_t st[8];
   unsigned cnt = 0;
-  for (int k = t; k < K; k += kSmThreads) {
-    const __half l = bias ? hadd(hb(z[k]), hb(bias[k])) : hb(z[k]);
-    uint16_t v = bh(hexp(hsub(l, m)));
+#pragma unroll
+  for (int i = 0; i < kSmMaxPer; ++i) {
+    if (t + i * kSmThreads >= K) break;
+    uint16_t v = bh(hexp(hsub(l[i], m)));
 #pragma unroll
     for (int lv = 0; lv < 8; ++lv) {
       if (cnt & (1u << lv)) {
@@ -2140,39 +2196,58 @@ __global__ void __launch_bounds__(kSmThreads)
     }
   ssum[t] = acc;
   __syncthreads();
-  for (int half = kSmThreads / 2; half >= 1; half /= 2) {
-    if (t < half) ssum[t] = bh(hadd(hb(ssum[t]), hb(ssum[t + half])));
-    __syncthreads();
-  }
-  if (t == 0) s_lse = hadd(m, hlog(hb(ssum[0])));
-  __syncthreads();
-  const __half lse = s_lse;
-  const int lab = labels[b];
-  for (int k = t; k < K; k += kSmThreads) {
-    const __half l = bias ? hadd(hb(z[k]), hb(bias[k])) : hb(z[k]);
-    __half p = hexp(hsub(l, lse));
+  // every warp closes the tree for itself: its levels of 32 and more from
+  // shared memory, the rest by shuffles
+  __half r[kWarps];
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) r[w] = hb(ssum[(t & 31) + 32 * w]);
+#pragma unroll
+  for (int half = kWarps / 2; half >= 1; half /= 2)
+#pragma unroll
+    for (int w = 0; w < half; ++w) r[w] = hadd(r[w], r[w + half]);
+  __half sum = r[0];
+#pragma unroll
+  for (int o = 16; o >= 1; o /= 2) sum = hadd(sum, hb((uint16_t)__shfl_down_sync(0xffffffffu, (unsigned)bh(sum), o)));
+  const __half lse =
+      hb((uint16_t)__shfl_sync(0xffffffffu, (unsigned)bh(hadd(m, hlog(sum))), 0));  // lane 0 holds the whole sum
+#pragma unroll
+  for (int i = 0; i < kSmMaxPer; ++i) {
+    const int k = t + i * kSmThreads;
+    if (k >= K) break;
+    __half p = hexp(hsub(l[i], lse));
     if (k == lab) {
       p = hsub(p, __float2half_rn(1.0f));
-      row_loss[b] = bh(hsub(lse, l));
+      row_loss[b] = bh(hsub(lse, l[i]));
     }
     dlogits[(long long)b * K + k] = bh(hmul(p, hb(invB)));
   }
 }
 
-__global__ void k_softmax_cols(const uint16_t* __restrict__ dlogits, const uint16_t* __restrict__ row_loss,
-                               int B, int K, int levels, uint16_t ratio, uint16_t* __restrict__ dbias,
-                               uint16_t* __restrict__ loss) {
+// CTAs 0 .. gridDim.x - 2: the column sums of 32 columns each (lane = column,
+// warp = an aligned run of 2^seg_levels rows, then the warps' nodes pairwise;
+// a missing right sibling passes its left one through, so the tree is that of
+// a row-by-row binary counter).  The last CTA: the batch mean of the row
+// losses, a halving tree over B padded to 2^levels.
+__global__ void __launch_bounds__(32 * kColSegs)
+    k_softmax_cols(const uint16_t* __restrict__ dlogits, const uint16_t* __restrict__ row_loss, int B, int K,
+                   int seg_levels, int levels, uint16_t ratio, uint16_t* __restrict__ dbias,
+                   uint16_t* __restrict__ loss) {
   pdl_wait();
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (dbias && k < K) {
-    uint16_t st[16];
+  __shared__ uint16_t node[kColSegs][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int seg = 1 << seg_levels;
+  if (blockIdx.x + 1 == gridDim.x) {
+    // thread t: the leaves [t * run, (t + 1) * run), run a power of two
+    const int run = levels > 10 ? 1 << (levels - 10) : 1;
+    uint32_t st[8];
     unsigned cnt = 0;
-    for (int b = 0; b < B; ++b) {
-      uint16_t v = dlogits[(long long)b * K + k];
+    for (int i = 0; i < run; ++i) {
+      const int b = threadIdx.x * run + i;
+      uint32_t v = b < B ? row_loss[b] : 0u;
 #pragma unroll
-      for (int lv = 0; lv < 16; ++lv) {
+      for (int lv = 0; lv < 8; ++lv) {
         if (cnt & (1u << lv)) {
-          v = bh(hadd(hb(st[lv]), hb(v)));
+          v = hmerge2(st[lv], v);
         } else {
           st[lv] = v;
           break;
@@ -2180,23 +2255,78 @@ __global__ void k_softmax_cols(const uint16_t* __restrict__ dlogits, const uint1
       }
       ++cnt;
     }
-    uint16_t acc = 0;
+    uint32_t acc = 0;
+#pragma unroll
+    for (int lv = 0; lv < 8; ++lv)
+      if (cnt == (1u << lv)) acc = st[lv];
+    // neighbouring threads, then neighbouring warps; `left` levels of the tree remain
+    int left = levels > 10 ? 10 : levels;
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const uint32_t other = __shfl_down_sync(0xffffffffu, acc, o);
+      if (left > 0) acc = hmerge2(acc, other);
+      --left;
+    }
+    if (lane == 0) node[w][0] = (uint16_t)acc;
+    __syncthreads();
+    if (w != 0) return;
+    acc = node[lane][0];
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const uint32_t other = __shfl_down_sync(0xffffffffu, acc, o);
+      if (left > 0) acc = hmerge2(acc, other);
+      --left;
+    }
+    if (lane == 0) *loss = (uint16_t)hmul2_rn(acc, dup2(ratio));
+    return;
+  }
+  const int k = blockIdx.x * 32 + lane;
+  const int b0 = w << seg_levels;
+  uint16_t st[12];
+  unsigned cnt = 0;
+  uint16_t acc = 0;
+  if (k < K) {
+    for (int i0 = 0; i0 < seg && b0 + i0 < B; i0 += 8) {
+      uint16_t q[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        q[i] = (i0 + i < seg && b0 + i0 + i < B) ? dlogits[(long long)(b0 + i0 + i) * K + k] : (uint16_t)0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (i0 + i >= seg || b0 + i0 + i >= B) break;
+        uint16_t v = q[i];
+#pragma unroll
+        for (int lv = 0; lv < 12; ++lv) {
+          if (cnt & (1u << lv)) {
+            v = bh(hadd(hb(st[lv]), hb(v)));
+          } else {
+            st[lv] = v;
+            break;
+          }
+        }
+        ++cnt;
+      }
+    }
     bool have = false;
 #pragma unroll
-    for (int lv = 0; lv < 16; ++lv)
+    for (int lv = 0; lv < 12; ++lv)
       if (cnt & (1u << lv)) {
         acc = have ? bh(hadd(hb(st[lv]), hb(acc))) : st[lv];
         have = true;
       }
-    dbias[k] = acc;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    // batch mean of the row losses: halving tree over B padded to 2^levels
-    Tree4<16, true> tree;
-    for (int b = 0; b < B; ++b) tree.push(make_uint4(row_loss[b], 0, 0, 0));
-    const uint4 acc = tree.finish(levels);
-    *loss = (uint16_t)hmul2_rn(acc.x, dup2(ratio));
+  node[w][lane] = acc;
+  __syncthreads();
+  // warp w closes column w: lane = segment
+  const int nseg = (B + seg - 1) >> seg_levels;
+  uint16_t v = node[lane][w];
+#pragma unroll
+  for (int o = 1; o < 32; o *= 2) {
+    const uint16_t other = (uint16_t)__shfl_down_sync(0xffffffffu, (unsigned)v, o);
+    if ((lane & (2 * o - 1)) == 0 && lane + o < nseg) v = bh(hadd(hb(v), hb(other)));
   }
+  const int kc = blockIdx.x * 32 + w;
+  if (lane == 0 && kc < K) dbias[kc] = v;
 }
 
 cudaError_t launch_softmax_xent(const uint16_t* logits, const uint16_t* bias,
@@ -2208,7 +2338,9 @@ cudaError_t launch_softmax_xent(const uint16_t* logits, const uint16_t* bias,
   while ((1 << L) < B) ++L;
   const uint16_t ratio = f16_bits_host((float)((double)(1 << L) / B));
   launch_pdl(k_softmax_rows, dim3(B), dim3(kSmThreads), 0, s, logits, bias, labels, K, invB, dlogits, ws);
-  launch_pdl(k_softmax_cols, dim3((K + 255) / 256), dim3(256), 0, s, dlogits, ws, B, K, L, ratio, dbias, loss);
+  const unsigned col_ctas = dbias ? (unsigned)((K + 31) / 32) : 0u;
+  launch_pdl(k_softmax_cols, dim3(col_ctas + 1), dim3(32 * kColSegs), 0, s, dlogits, ws, B, K, std::max(0, L - 5), L,
+             ratio, dbias, loss);
   return counted_launches(2);
 }
 
