@@ -181,6 +181,19 @@ int pick_bn_out(long long n) {  // tile width for an output of n columns
   if (n % 256 == 0 || n > 192) return 256;
   return 192;
 }
+// Narrower tiles while they leave every tile an SM of its own: with fewer tiles
+// than SMs a launch lasts as long as one tile, and halving its width takes the
+// K-block from ~500 to ~270 (128) and ~180 (64) cycles of MMA and half of its
+// weight traffic off that chain.  The classifier's forward at batch 256 (8
+// tiles of 256, 32 K-blocks each): 22.4 -> 18.4 us with 32 tiles of 64, its
+// data gradient 16.3 -> 12.3 us.  The rule stops where the tiles would outnumber the SMs (a second round costs
+// more than it saves), so a fused-statistics launch keeps one tile, hence one
+// slot, per M tile and the same statistics tree.
+int fill_bn(int bn, long long m_tiles, long long n, int sms) {
+  for (int half : {128, 64})
+    if (half < bn && m_tiles * ((n + half - 1) / half) <= sms) bn = half;
+  return bn;
+}
 int pick_bn_wgrad(long long n) {
   if (n % 256 == 0) return 256;
   if (n % 192 == 0) return 192;
@@ -562,6 +575,7 @@ int run_dgrad_phases(const Shape& s, const uint16_t* dy, const uint16_t* w, uint
   CUtensorMap ma, mb;
   p.M = (int)(s.N * gh * gw);
   p.N = (int)s.C;
+  BN = fill_bn(BN, 4ll * cdiv(p.M, kBM), s.C, sms);
   p.a_mode = LD_IM2COL_K;
   p.b_mode = LD_TAP3D_MN;
   set_kmajor(p, true, false);
@@ -902,7 +916,7 @@ static int conv_fwd_impl(const pf16_conv_desc* d, const uint16_t* x, const uint1
   if (const int ws_s2d = stem_s2d_width(s, (flags & PF16_ACCUMULATE) != 0))
     return run_stem_s2d(s, ws_s2d, x, w, y, ws, status, sms, st, stats, f32);
   set_stats(p, stats, s.K);
-  const int BN = pick_bn_out(s.K);
+  const int BN = fill_bn(pick_bn_out(s.K), cdiv(p.M, kBM), s.K, sms);
   p.a_mode = LD_TILED_K;
   p.b_mode = LD_TILED_K;
   set_kmajor(p, true, true);
@@ -1004,7 +1018,7 @@ static int conv_dgrad_impl(const pf16_conv_desc* d, const uint16_t* dy, const ui
     return run_halo(s, ws, true, dy, w, dx, status, sms, st, f32, stats, stats ? bn : nullptr);
   // with an addend the TMA-fed epilogue leaves 256-wide tiles two pipeline
   // stages; reductions of 4+ K-blocks keep three with 128-wide tiles
-  const int BN = (add && s.K >= 4 * kBK) ? std::min(pick_bn_out(s.C), 128) : pick_bn_out(s.C);
+  const int bn_max = (add && s.K >= 4 * kBK) ? std::min(pick_bn_out(s.C), 128) : pick_bn_out(s.C);
   const size_t dx_elems = (size_t)(s.N * s.H * s.W * s.C);
 
   if (s.R == 1 && s.S == 1 && s.pad == 0) {
@@ -1018,6 +1032,7 @@ static int conv_dgrad_impl(const pf16_conv_desc* d, const uint16_t* dy, const ui
     CUtensorMap ma, mb;
     p.M = (int)(s.N * s.P * s.Q);
     p.N = (int)s.C;
+    const int BN = fill_bn(bn_max, cdiv(p.M, kBM), s.C, sms);
     p.a_mode = LD_TILED_K;
     p.b_mode = LD_TILED_MN;
     set_kmajor(p, true, false);
@@ -1046,7 +1061,7 @@ static int conv_dgrad_impl(const pf16_conv_desc* d, const uint16_t* dy, const ui
   bool any_empty = false;
   for (int ph = 0; ph < s.st; ++ph)
     for (int pw = 0; pw < s.st; ++pw) any_empty |= make_phase(s, ph, pw).empty();
-  if (phases_one_launch(s)) return run_dgrad_phases(s, dy, w, dx, status, sms, st, f32, accum, BN, stats, bn);
+  if (phases_one_launch(s)) return run_dgrad_phases(s, dy, w, dx, status, sms, st, f32, accum, bn_max, stats, bn);
   if (any_empty && !accum && launch_fill_zero(dx, dx_elems, st) != cudaSuccess)
     return PF16_ERR_CUDA;
   for (int ph = 0; ph < s.st; ++ph)
@@ -1063,6 +1078,7 @@ static int conv_dgrad_impl(const pf16_conv_desc* d, const uint16_t* dy, const ui
       CUtensorMap ma, mb;
       p.M = (int)(s.N * gh * gw);
       p.N = (int)s.C;
+      const int BN = fill_bn(bn_max, cdiv(p.M, kBM), s.C, sms);
       p.a_mode = LD_IM2COL_K;
       p.b_mode = LD_TAP3D_MN;
       set_kmajor(p, true, false);
