@@ -62,7 +62,7 @@ __device__ __forceinline__ void grid_decompose(int m, const PixGrid& g, int& n, 
 // Producer state of one work unit: everything that depends only on the tile
 // is decomposed once, and the per-K-block coordinates advance incrementally
 // (no integer divisions on the single issuing thread's critical path).
-template <int BN>
+template <int BN, int AM, int BM>
 struct Cursor {
   int kb;
   // A, im2col: input coordinates of the tile's first pixel; current tap / chunk
@@ -76,7 +76,7 @@ struct Cursor {
 
   __device__ __forceinline__ void init(const GemmParams& p, int m0, int n0, int kb0) {
     kb = kb0;
-    if (p.a_mode == LD_IM2COL_K) {
+    if constexpr (AM == LD_IM2COL_K) {
       int n, i, j;
       grid_decompose(m0, p.ga, n, i, j);
       a_w = j * p.ga.step + p.ga.base_w;
@@ -85,7 +85,7 @@ struct Cursor {
       a_tap = kb0 / p.a_cpt;
       a_c = (kb0 - a_tap * p.a_cpt) * 64;
     }
-    if (p.b_mode == LD_IM2COL_MN) {
+    if constexpr (BM == LD_IM2COL_MN) {
       grid_decompose(kb0 * kBK, p.gb, b_n, b_i, b_j);
 #pragma unroll
       for (int j = 0; j < BN / 64; ++j) {
@@ -100,7 +100,7 @@ struct Cursor {
         b_c[j] = c0;
       }
     }
-    if (p.b_mode == LD_TAP3D_MN) {
+    if constexpr (BM == LD_TAP3D_MN) {
       b_t = kb0 / p.b_cpt;
       b_k = (kb0 - b_t * p.b_cpt) * 64;
     }
@@ -108,14 +108,14 @@ struct Cursor {
 
   __device__ __forceinline__ void advance(const GemmParams& p) {
     ++kb;
-    if (p.a_mode == LD_IM2COL_K) {
+    if constexpr (AM == LD_IM2COL_K) {
       a_c += 64;
       if (a_c == p.a_cpt * 64) {
         a_c = 0;
         ++a_tap;
       }
     }
-    if (p.b_mode == LD_IM2COL_MN) {
+    if constexpr (BM == LD_IM2COL_MN) {
       b_j += kBK;
       while (b_j >= p.gb.gw) {
         b_j -= p.gb.gw;
@@ -125,7 +125,7 @@ struct Cursor {
         }
       }
     }
-    if (p.b_mode == LD_TAP3D_MN) {
+    if constexpr (BM == LD_TAP3D_MN) {
       b_k += 64;
       if (b_k == p.b_cpt * 64) {
         b_k = 0;
@@ -137,47 +137,30 @@ struct Cursor {
   // the K-block's A and B boxes into stage (sa, sb), completing on bar
   __device__ __forceinline__ void load(const GemmParams& p, const CUtensorMap* ma, const CUtensorMap* mb,
                                        uint32_t sa, uint32_t sb, uint32_t bar, int m0, int n0) const {
-    switch (p.a_mode) {
-      case LD_TILED_K:
-        tma_load_2d(sa, ma, bar, kb * kBK, m0);
-        break;
-      case LD_TILED_MN:
-        tma_load_2d(sa, ma, bar, m0, kb * kBK);
-        tma_load_2d(sa + 8192, ma, bar, m0 + 64, kb * kBK);
-        break;
-      case LD_IM2COL_K:
-        tma_load_im2col_4d(sa, ma, bar, a_c, a_w, a_h, a_n, (uint16_t)p.tap_ds[a_tap],
-                           (uint16_t)p.tap_dr[a_tap]);
-        break;
-      default:
-        break;
+    if constexpr (AM == LD_TILED_K) {
+      tma_load_2d(sa, ma, bar, kb * kBK, m0);
+    } else if constexpr (AM == LD_TILED_MN) {
+      tma_load_2d(sa, ma, bar, m0, kb * kBK);
+      tma_load_2d(sa + 8192, ma, bar, m0 + 64, kb * kBK);
+    } else {
+      static_assert(AM == LD_IM2COL_K, "A's load modes");
+      tma_load_im2col_4d(sa, ma, bar, a_c, a_w, a_h, a_n, (uint16_t)p.tap_ds[a_tap], (uint16_t)p.tap_dr[a_tap]);
     }
-    switch (p.b_mode) {
-      case LD_TILED_K:
-        tma_load_2d(sb, mb, bar, kb * kBK, n0);
-        break;
-      case LD_TILED_MN:
+    if constexpr (BM == LD_TILED_K) {
+      tma_load_2d(sb, mb, bar, kb * kBK, n0);
+    } else if constexpr (BM == LD_TILED_MN) {
 #pragma unroll
-        for (int j = 0; j < BN / 64; ++j) {
-          tma_load_2d(sb + j * 8192, mb, bar, n0 + 64 * j, kb * kBK);
-        }
-        break;
-      case LD_IM2COL_MN: {
-        const int bw = b_j * p.gb.step + p.gb.base_w, bh = b_i * p.gb.step + p.gb.base_h;
+      for (int j = 0; j < BN / 64; ++j) tma_load_2d(sb + j * 8192, mb, bar, n0 + 64 * j, kb * kBK);
+    } else if constexpr (BM == LD_IM2COL_MN) {
+      const int bw = b_j * p.gb.step + p.gb.base_w, bh = b_i * p.gb.step + p.gb.base_h;
 #pragma unroll
-        for (int j = 0; j < BN / 64; ++j) {
-          tma_load_im2col_4d(sb + j * 8192, mb, bar, b_c[j], bw, bh, b_n, (uint16_t)p.tap_ds[b_tap[j]],
-                             (uint16_t)p.tap_dr[b_tap[j]]);
-        }
-      } break;
-      case LD_TAP3D_MN:
+      for (int j = 0; j < BN / 64; ++j)
+        tma_load_im2col_4d(sb + j * 8192, mb, bar, b_c[j], bw, bh, b_n, (uint16_t)p.tap_ds[b_tap[j]],
+                           (uint16_t)p.tap_dr[b_tap[j]]);
+    } else {
+      static_assert(BM == LD_TAP3D_MN, "B's load modes");
 #pragma unroll
-        for (int j = 0; j < BN / 64; ++j) {
-          tma_load_3d(sb + j * 8192, mb, bar, n0 + 64 * j, p.tap_w[b_t], b_k);
-        }
-        break;
-      default:
-        break;
+      for (int j = 0; j < BN / 64; ++j) tma_load_3d(sb + j * 8192, mb, bar, n0 + 64 * j, p.tap_w[b_t], b_k);
     }
   }
 };
@@ -198,6 +181,65 @@ __device__ __forceinline__ void unit_decode(const GemmParams& p, int u, int& m0,
   } else {
     kb0 = split * p.kb_per_split;
     kb1 = min(p.num_kb, kb0 + p.kb_per_split);
+  }
+}
+
+// The TMA producer (one thread): the K-blocks of the CTA's units into the ring
+// of stages.  An SM takes 48 KB (a 128-row and a 256-row box) by TMA in ~410
+// cycles, less than the K-block's ~500 cycles of MMA, so what bounds the ring is
+// this thread's instruction path: with the modes tested per K-block and plain
+// lane predication a stage took 560 (two boxes) to 1,000 cycles (five), and
+// every im2col GEMM was bound by it.  Hence the load modes are compile-time and
+// the thread is an elected one (elect_one), here and in the MMA role.  3x3,
+// 28x28, 128 -> 128 at batch 256: forward 69.0 -> 46.5 us, data gradient 78.6
+// -> 48.4 us; 27x27, 192 -> 320 at batch 13: weight gradient 25.7 -> 17.7 us.
+struct ProducerArgs {
+  const CUtensorMap *ma, *mb;
+  uint8_t* smem;
+  uint64_t *full, *empty;
+  volatile int* abort_flag;
+  int cid, ncl, total;
+  uint64_t lim;
+};
+template <int BN, class Cfg, int AM, int BM>
+__device__ __forceinline__ void produce(const GemmParams& p, const ProducerArgs& a) {
+  int stage = 0;
+  uint32_t phase = 0;
+  uint32_t issued = 0;  // stages loaded so far (for the drain below)
+  for (int u = a.cid; u < a.total && !*a.abort_flag; u += a.ncl) {
+    int m0, n0, split, kb0, kb1;
+    unit_decode(p, u, m0, n0, split, kb0, kb1, BN);
+    Cursor<BN, AM, BM> cur;
+    cur.init(p, m0, n0, kb0);
+    for (int kb = kb0; kb < kb1; ++kb, cur.advance(p)) {
+      if (!mbar_wait(smem_u32(&a.empty[stage]), phase ^ 1, a.lim)) {
+        record_timeout(p, a.abort_flag);
+        break;
+      }
+      const uint32_t sa = smem_u32(a.smem + stage * Cfg::STAGE_BYTES);
+      const uint32_t fb = smem_u32(&a.full[stage]);
+      mbar_arrive_expect_tx(fb, Cfg::STAGE_BYTES);
+      cur.load(p, a.ma, a.mb, sa, sa + Cfg::A_BYTES, fb, m0, n0);
+      ++issued;
+      if (++stage == Cfg::STAGES) {
+        stage = 0;
+        phase ^= 1;
+      }
+    }
+  }
+  if (*a.abort_flag) {
+    // Another role gave up: let the copies this thread started land before
+    // the CTA's shared memory is released (each wait bounded on its own).
+    const uint32_t n = issued < (uint32_t)Cfg::STAGES ? issued : (uint32_t)Cfg::STAGES;
+    int s = stage;
+    uint32_t ph = phase;
+    for (uint32_t i = 0; i < n; ++i) {
+      if (--s < 0) {
+        s = Cfg::STAGES - 1;
+        ph ^= 1;
+      }
+      mbar_wait(smem_u32(&a.full[s]), ph, 1000000000ull);
+    }
   }
 }
 
@@ -588,48 +630,25 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
   const uint64_t lim = p.wait_limit_ns;
 
   if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t issued = 0;  // stages loaded so far (for the drain below)
-      for (int u = cid; u < total && !*abort_flag; u += ncl) {
-        int m0, n0, split, kb0, kb1;
-        unit_decode(p, u, m0, n0, split, kb0, kb1, BN);
-        Cursor<BN> cur;
-        cur.init(p, m0, n0, kb0);
-        for (int kb = kb0; kb < kb1; ++kb, cur.advance(p)) {
-          if (!mbar_wait(smem_u32(&empty[stage]), phase ^ 1, lim)) {
-            record_timeout(p, abort_flag);
-            break;
-          }
-          const uint32_t sa = smem_u32(smem + stage * Cfg::STAGE_BYTES);
-          const uint32_t fb = smem_u32(&full[stage]);
-          mbar_arrive_expect_tx(fb, Cfg::STAGE_BYTES);
-          cur.load(p, &mapA, &mapB, sa, sa + Cfg::A_BYTES, fb, m0, n0);
-          ++issued;
-          if (++stage == Cfg::STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
-        }
-      }
-      if (*abort_flag) {
-        // Another role gave up: let the copies this thread started land before
-        // the CTA's shared memory is released (each wait bounded on its own).
-        const uint32_t n = issued < (uint32_t)Cfg::STAGES ? issued : (uint32_t)Cfg::STAGES;
-        int s = stage;
-        uint32_t ph = phase;
-        for (uint32_t i = 0; i < n; ++i) {
-          if (--s < 0) {
-            s = Cfg::STAGES - 1;
-            ph ^= 1;
-          }
-          mbar_wait(smem_u32(&full[s]), ph, 1000000000ull);
-        }
-      }
+    if (elect_one()) {
+      // the load modes are compile-time in each of the six pairs the plans use
+      const ProducerArgs a{&mapA, &mapB, smem, full, empty, abort_flag, cid, ncl, total, lim};
+      const int am = p.a_mode, bm = p.b_mode;
+      if (am == LD_TILED_K && bm == LD_TILED_K)
+        produce<BN, Cfg, LD_TILED_K, LD_TILED_K>(p, a);
+      else if (am == LD_IM2COL_K && bm == LD_TILED_K)
+        produce<BN, Cfg, LD_IM2COL_K, LD_TILED_K>(p, a);
+      else if (am == LD_TILED_K && bm == LD_TILED_MN)
+        produce<BN, Cfg, LD_TILED_K, LD_TILED_MN>(p, a);
+      else if (am == LD_IM2COL_K && bm == LD_TAP3D_MN)
+        produce<BN, Cfg, LD_IM2COL_K, LD_TAP3D_MN>(p, a);
+      else if (am == LD_TILED_MN && bm == LD_TILED_MN)
+        produce<BN, Cfg, LD_TILED_MN, LD_TILED_MN>(p, a);
+      else
+        produce<BN, Cfg, LD_TILED_MN, LD_IM2COL_MN>(p, a);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
@@ -1175,7 +1194,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   const uint64_t lim = p.wait_limit_ns;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // resident weights: the 64-row slice of each tap
       const uint32_t bb = smem_u32(bready);
       mbar_arrive_expect_tx(bb, (uint32_t)(NTAPS * B_TILE));
@@ -1220,7 +1239,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = mbar_wait(smem_u32(bready), 0, lim);
       if (!ok) record_timeout(p, abort_flag);
       tc_fence_after();
@@ -1498,7 +1517,7 @@ __global__ void __launch_bounds__(kStemWgradThreads, 1)
   const uint64_t lim = p.wait_limit_ns;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0, issued = 0;
       for (int c = blockIdx.x; c < chunks && !*abort_flag; c += gridDim.x) {
@@ -1535,7 +1554,7 @@ __global__ void __launch_bounds__(kStemWgradThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // A: dy, MN-major 128-byte swizzle, M atoms one padded row (ws * 128 B)
       // apart, 8-pixel K groups 1 KB apart; B: xs, MN-major 32-byte swizzle,
       // N atoms one pixel (32 B) apart, 8-pixel K groups 256 B apart
@@ -1730,7 +1749,7 @@ __global__ void __launch_bounds__(kWgrad3Threads, 1)
   const uint64_t lim = p.wait_limit_ns;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0, issued = 0;
       for (int c = blockIdx.x; c < chunks && !*abort_flag; c += gridDim.x) {
@@ -1767,7 +1786,7 @@ __global__ void __launch_bounds__(kWgrad3Threads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // A: dy, MN-major 128-byte swizzle, M atoms one padded row apart, 8-pixel
       // K groups 1 KB apart; B: the input, three N atoms one pixel apart
       const uint64_t adesc0 = smem_desc(0, Cfg::WS * 128, 1024, 2);

@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   const uint64_t lim = p.wait_limit_ns;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int as = 0, bs = 0;
       uint32_t aph = 0, bph = 0, a_issued = 0, b_issued = 0;
       bool ok = true;
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       int as = 0, bs = 0, acc = 0;
       uint32_t aph = 0, bph = 0, acc_phase = 0;
       // tap windows in 16-byte units, and the two base descriptors
@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(kWideWgradThreads, 1)
   const uint64_t lim = p.wait_limit_ns;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0, issued = 0;
       bool ok = true;
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kWideWgradThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // A: dy, MN-major, two 64-channel atoms 16 KB apart, 8-pixel K groups
       // 1 KB apart; B: the input, three 64-channel atoms one pixel apart
       const uint64_t adesc0 = smem_desc(0, 16384, 1024, 2);
