@@ -236,13 +236,14 @@ WgradSplit wgrad_split(const Shape& s) {
   double best = -1.0;
   w.kb_per_split = std::min(w.num_kb, 64);
   w.splits = cdiv(w.num_kb, w.kb_per_split);
-  for (int sp = 1; sp <= 1024; ++sp) {
-    const int kps = cdiv(w.num_kb, sp);
-    if (kps > 64) continue;
-    if (kps < 4 && sp > 1) break;  // kps only shrinks from here
+  // chunk lengths in falling order, each the shortest with its split count (every
+  // split count up to 1024 has such a length): at most 61 candidates a call
+  const int kps_min = std::max(4, cdiv(w.num_kb, 1024));
+  for (int kps = std::min(64, w.num_kb); kps >= std::min(kps_min, w.num_kb) && kps > 0; --kps) {
     const int real = cdiv(w.num_kb, kps);
-    const long long rounds = (tiles * real + kPlanSms - 1) / kPlanSms;
-    const double t = (double)rounds * (kps * t_kb + t_unit) + (real > 1 ? real * dw_bytes * 2.0 / kPartialBw : 0.0);
+    if (real > 1024 || cdiv(w.num_kb, real) != kps) continue;
+    const double rounds = (double)((tiles * real + kPlanSms - 1) / kPlanSms);
+    const double t = rounds * (kps * t_kb + t_unit) + (real > 1 ? real * dw_bytes * 2.0 / kPartialBw : 0.0);
     if (best < 0.0 || t < best * (1.0 - 1e-9)) {
       best = t;
       w.kb_per_split = kps;

@@ -82,6 +82,9 @@ class BnTensors(ctypes.Structure):
     _fields_ = [(n, ctypes.c_void_p) for n in _BN_T]
 
 
+_BN_FIELDS = frozenset(_BN_T)
+
+
 _lock = threading.Lock()
 _lib = None
 
@@ -89,6 +92,8 @@ _lib = None
 def lib():
     """Load (building first if needed) libpf16.so."""
     global _lib
+    if _lib is not None:  # loaded: calls on the hot path take no lock
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build()
@@ -157,7 +162,7 @@ def lib():
             L.pf16_device_arch.restype = I
             L.pf16_kernel_launches.argtypes = []
             L.pf16_kernel_launches.restype = ctypes.c_uint64
-            _lib = L
+            _lib = L  # last: other threads may use it from here on
     return _lib
 
 
@@ -170,24 +175,34 @@ def _check(rc: int, where: str) -> None:
         raise PF16Error(rc, where)
 
 
+# Every call passes through these, and the smallest kernels take less time than
+# the marshalling of their arguments: plain ints (ctypes converts them to the
+# declared void pointers itself), and the current stream's handle without a
+# Stream object around it.
 def _ptr(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = None
 
 
 def _stream(stream):
+    global _raw_stream
     if stream is None:
-        import torch
+        if _raw_stream is None:
+            import torch
 
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+            torch.cuda.init()
+            get, dev = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+            _raw_stream = lambda: get(dev())
+        return _raw_stream()
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _nbytes(t):
-    return 0 if t is None else t.numel() * t.element_size()
+    return 0 if t is None else t.nbytes
 
 
 def conv_desc(n, h, w, c, k, r, s, stride, pad) -> ConvDesc:
@@ -299,8 +314,18 @@ def bn_workspace_size(d: BnDesc) -> int:
     return int(lib().pf16_bn_workspace_size(ctypes.byref(d)))
 
 
+def _bn_tensors(tensors):
+    t = BnTensors()
+    for k, v in tensors.items():
+        if k not in _BN_FIELDS:
+            raise TypeError(f"unexpected BatchNorm tensor {k!r}")
+        if v is not None:
+            setattr(t, k, v.data_ptr())
+    return t
+
+
 def bn_fwd_bwd(d, phase, ws, stream=None, **tensors):
-    t = BnTensors(**{k: (v.data_ptr() if v is not None else None) for k, v in tensors.items()})
+    t = _bn_tensors(tensors)
     _check(lib().pf16_bn_fwd_bwd(ctypes.byref(d), phase, ctypes.byref(t), _ptr(ws), _nbytes(ws),
                                  _stream(stream)), "pf16_bn_fwd_bwd")
 
@@ -308,7 +333,7 @@ def bn_fwd_bwd(d, phase, ws, stream=None, **tensors):
 def bn_relu_maxpool_fwd(d, ws, pooled, argmax, stream=None, **tensors):
     """The stem's BatchNorm (phase 0, ReLU) with its output max-pooled at once;
     y is not stored (pass no y).  tensors as bn_fwd_bwd's."""
-    t = BnTensors(**{k: (v.data_ptr() if v is not None else None) for k, v in tensors.items()})
+    t = _bn_tensors(tensors)
     _check(lib().pf16_bn_relu_maxpool_fwd(ctypes.byref(d), ctypes.byref(t), _ptr(pooled), _ptr(argmax), _ptr(ws),
                                           _nbytes(ws), _stream(stream)), "pf16_bn_relu_maxpool_fwd")
 
