@@ -647,19 +647,18 @@ __device__ __forceinline__ uint4 and4(uint4 a, uint4 m) {
 __device__ __forceinline__ uint4 relu_mask4(uint4 y) {
   return make_uint4(relu_mask2(y.x), relu_mask2(y.y), relu_mask2(y.z), relu_mask2(y.w));
 }
-// the two lane bits of a per-lane all-ones mask
-__device__ __forceinline__ uint32_t mask_bits2(uint32_t m) { return (m & 1u) | ((m >> 15) & 2u); }
-// ReLU of z, and the decisions as bits (bit j: lane j of z is > 0)
+// ReLU of z, and the decisions as bits (bit j: lane j of z is > 0): a byte of
+// each half's mask, the byte's own bit of it, and the four bytes summed
 __device__ __forceinline__ uint4 relu_bits(uint4 z, uint32_t& bits) {
   const uint4 m = relu_mask4(z);
-  bits = mask_bits2(m.x) | mask_bits2(m.y) << 2 | mask_bits2(m.z) << 4 | mask_bits2(m.w) << 6;
+  const uint32_t lo = prmt(m.x, m.y, 0x6420u) & 0x08040201u, hi = prmt(m.z, m.w, 0x6420u) & 0x80402010u;
+  bits = ((lo | hi) * 0x01010101u) >> 24;
   return and4(z, m);
 }
-__device__ __forceinline__ uint32_t bits_mask2(uint32_t b) {
-  return ((b & 1u) ? 0x0000FFFFu : 0u) | ((b & 2u) ? 0xFFFF0000u : 0u);
-}
+// bits back to per-lane all-ones masks (b < 256)
 __device__ __forceinline__ uint4 bits_mask4(uint32_t b) {
-  return make_uint4(bits_mask2(b), bits_mask2(b >> 2), bits_mask2(b >> 4), bits_mask2(b >> 6));
+  const uint2 lo = bits_mask_4(b), hi = bits_mask_4(b >> 4);
+  return make_uint4(lo.x, lo.y, hi.x, hi.y);
 }
 
 // Combination of (mean, variance) pairs by the pairwise parallel variance
@@ -1875,27 +1874,22 @@ cudaError_t launch_maxpool_bwd(const uint16_t* x, const uint16_t* dy, uint16_t* 
 // starts from its first valid cell and replaces the maximum where a cell is
 // strictly greater (set.gt on f16x2, exact for these values): the pooled
 // output and positions are those of k_maxpool_fwd on y, bit for bit.
+// Bound by issue (ncu at batch 128: 67% of the slots at 34% of the warps), so
+// the decisions are native compares and positions stay 16-bit lanes until a
+// window is done.
 // ============================================================================
 constexpr int kBpT = 2;
 
-__device__ __forceinline__ uint32_t hgt2_mask(uint32_t a, uint32_t b) {  // 0xFFFF per half where a > b
-  uint32_t d;
-  asm("set.gt.u32.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-
-// take cell value v (position rs) into the window's running maximum m / codes
-__device__ __forceinline__ void pool_take(uint4& m, uint32_t (&code)[2], const uint4& v, uint32_t rs) {
-  const uint32_t rsr = rs * 0x01010101u;
-  uint32_t* mw = &m.x;
+// take cell value v (position rs in each half) into the window's running
+// maximum m and positions (one 16-bit lane per channel until the window is done)
+__device__ __forceinline__ void pool_take(uint4& m, uint4& code, const uint4& v, uint32_t rs) {
+  uint32_t *mw = &m.x, *cw = &code.x;
   const uint32_t* vw = &v.x;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const uint32_t gt = hgt2_mask(vw[k], mw[k]);
     mw[k] = (vw[k] & gt) | (mw[k] & ~gt);
-    // the position bytes of halves 2k, 2k+1: bytes 2(k&1), 2(k&1)+1 of code word k/2
-    const uint32_t bm = __byte_perm(gt, 0u, 0x4420) << (16 * (k & 1));
-    code[k >> 1] = (code[k >> 1] & ~bm) | (rsr & bm);
+    cw[k] = (rs & gt) | (cw[k] & ~gt);
   }
 }
 
@@ -1966,8 +1960,8 @@ __global__ void __launch_bounds__(256)
       // the window's first valid cell (row 2p - 1 and column 2q - 1 are padding at p = 0, q = 0)
       const int r0 = p == 0 ? 1 : 0, s0 = q == 0 ? 1 : 0;
       uint4 m = zs[((2 * t + r0) * W + 2 * q + s0 - 1) * tc + cg];
-      uint32_t code[2];
-      code[0] = code[1] = (uint32_t)(r0 * 3 + s0) * 0x01010101u;
+      const uint32_t first = (uint32_t)(r0 * 3 + s0) * 0x00010001u;
+      uint4 code = make_uint4(first, first, first, first);
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
         if (2 * p + r - 1 >= H || r < r0) continue;
@@ -1975,12 +1969,13 @@ __global__ void __launch_bounds__(256)
         for (int s2 = 0; s2 < 3; ++s2) {
           const int w = 2 * q + s2 - 1;
           if (w < 0 || w >= W || (r == r0 && s2 <= s0)) continue;
-          pool_take(m, code, zs[((2 * t + r) * W + w) * tc + cg], (uint32_t)(r * 3 + s2));
+          pool_take(m, code, zs[((2 * t + r) * W + w) * tc + cg], (uint32_t)(r * 3 + s2) * 0x00010001u);
         }
       }
       const long long o = (((long long)n * P + p) * Q + q) * tc + cg;
       reinterpret_cast<uint4*>(pooled)[o] = m;
-      reinterpret_cast<uint2*>(codes)[o] = make_uint2(code[0], code[1]);
+      reinterpret_cast<uint2*>(codes)[o] =
+          make_uint2(prmt(code.x, code.y, 0x6420u), prmt(code.z, code.w, 0x6420u));
     }
   }
 }

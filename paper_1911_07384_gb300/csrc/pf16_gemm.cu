@@ -422,14 +422,11 @@ __device__ __forceinline__ void epilogue_bs(const GemmParams& p, const CUtensorM
         uint4 a;
         ld_shared_v4(addr, a);
         const uint32_t bits = ((j < 4 ? cur.am.x : cur.am.y) >> (8 * (j & 3))) & 0xFFu;
-        uint32_t mk[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mk[k] = (((bits >> (2 * k)) & 1u) ? 0x0000FFFFu : 0u) | (((bits >> (2 * k + 1)) & 1u) ? 0xFFFF0000u : 0u);
-        v.x = hadd2_rn(v.x, a.x & mk[0]);
-        v.y = hadd2_rn(v.y, a.y & mk[1]);
-        v.z = hadd2_rn(v.z, a.z & mk[2]);
-        v.w = hadd2_rn(v.w, a.w & mk[3]);
+        const uint2 mlo = bits_mask_4(bits), mhi = bits_mask_4(bits >> 4);
+        v.x = hadd2_rn(v.x, a.x & mlo.x);
+        v.y = hadd2_rn(v.y, a.y & mlo.y);
+        v.z = hadd2_rn(v.z, a.z & mhi.x);
+        v.w = hadd2_rn(v.w, a.w & mhi.y);
       }
       st_shared_v4(addr, v);
     }

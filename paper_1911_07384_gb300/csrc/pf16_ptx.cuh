@@ -273,10 +273,27 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, bool a_mn, bool b
 // Exact binary16 arithmetic: one IEEE roundTiesToEven rounding per op, never
 // contracted into an FMA, subnormals kept (no .ftz).
 // ----------------------------------------------------------------------------
-// per-lane all-ones where the binary16 lane is > 0 and not NaN: as an unsigned
-// 16-bit code h, 1 <= h <= 0x7C00, i.e. (h - 1) < 0x7C00 -- two SIMD ops
-__device__ __forceinline__ uint32_t relu_mask2(uint32_t y) {
-  return __vcmpltu2(__vsub2(y, 0x00010001u), 0x7C007C00u);
+// 0xFFFF per half where a > b (false for NaN; subnormals compare exactly)
+__device__ __forceinline__ uint32_t hgt2_mask(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("set.gt.u32.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// the ReLU's decision: 0xFFFF per half where it is > 0 and not NaN.  One
+// compare: the halfword SIMD forms (vsub2, vcmpltu2) are emulated in about a
+// dozen instructions, and took a third of the BatchNorm apply's issue slots.
+__device__ __forceinline__ uint32_t relu_mask2(uint32_t y) { return hgt2_mask(y, 0u); }
+// byte permutation; a selector nibble of 8 + i fills its byte with byte i's sign bit
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
+}
+// the low four bits of b as all-ones halves: bit i goes to byte i's sign bit
+// (the shifted copies of a 4-bit value do not meet), which prmt spreads
+__device__ __forceinline__ uint2 bits_mask_4(uint32_t b) {
+  const uint32_t t = (b & 15u) * 0x10204080u;
+  return make_uint2(prmt(t, 0u, 0x9988u), prmt(t, 0u, 0xBBAAu));
 }
 __device__ __forceinline__ uint32_t hadd2_rn(uint32_t a, uint32_t b) {
   uint32_t d;
