@@ -1635,7 +1635,9 @@ __device__ __forceinline__ uint32_t heq2_mask(uint32_t a, uint32_t b) {  // 0xFF
 // thread owns that 2x2 block of cells for one group of 8 channels: it loads
 // the four windows' positions and gradients once, then every cell sums, in
 // window order (p, then q), the gradients of the windows whose first maximum
-// it is.  One CTA per block row (n, i).
+// it is.  One CTA per block row (n, i).  Bound by issue (64% of the slots at batch
+// 128): the masked gradients are added without a test of the mask (56.8 -> 54.3
+// us at 128 x 112 x 112 x 64, 7.5 -> 6.7 us at 32 x 80 x 80 x 64).
 __global__ void __launch_bounds__(512)
     k_maxpool_bwd_codes(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ dy,
                         uint16_t* __restrict__ dx, int N, int H, int W, int C, int P, int Q) {
@@ -1689,8 +1691,8 @@ __global__ void __launch_bounds__(512)
             const uint32_t* gw = reinterpret_cast<const uint32_t*>(&g[a][b]);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const uint32_t sel = heq2_mask(cw16[a][b][k], mine);
-              if (sel) acc[k] = hadd2_rn(acc[k], gw[k] & sel);
+              // (a +0 where another cell was the maximum: the sum never is -0)
+              acc[k] = hadd2_rn(acc[k], gw[k] & heq2_mask(cw16[a][b][k], mine));
             }
           }
         }
