@@ -416,7 +416,7 @@ cudaError_t launch_gemm_halo_wide(int BN, const CUtensorMap& mA, const CUtensorM
 // meets a real input pixel (column 0 of the next image), so an infinite or
 // NaN input there gives NaN in the s = 2 taps.
 // Roles: warp 0 the TMA producer, warp 1 the TMEM owner and MMA issuer,
-// warps 2-5 the epilogue (TMEM sub-partition warp % 4).  Every mbarrier wait
+// warps 2-9 the epilogue (TMEM sub-partition warp % 4).  Every mbarrier wait
 // is bounded; on expiry the CTA records PF16_ERR_TIMEOUT and all roles leave.
 // ---------------------------------------------------------------------------
 struct WideWgradCfg {
@@ -431,7 +431,11 @@ struct WideWgradCfg {
   static_assert(STAGE % 1024 == 0, "stage bases keep the 1024-byte alignment of the 128-byte swizzle");
   static_assert(SMEM <= 232448, "shared memory per CTA");
 };
-constexpr int kWideWgradThreads = 192;
+// 8 epilogue warps, two per TMEM sub-partition, halve the drain that a CTA's last
+// unit exposes, and only the rows that no copy writes are cleared at the start
+// (14x14, 256-256 at batch 64 17.2 -> 16.4 us with the split-K tree, 7x7, 512-512 at
+// batch 256 47.3 -> 46.4 us)
+constexpr int kWideWgradThreads = 320;
 
 // Unit u: chunk q = u / types, then filter row r, input chunk cc and
 // output-channel tile kt (r fastest).
@@ -469,9 +473,18 @@ __global__ void __launch_bounds__(kWideWgradThreads, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // zero the stages once: rows past a box are never written by a copy
-  for (int i = threadIdx.x; i < Cfg::STAGES * Cfg::STAGE / 16; i += blockDim.x)
-    st_shared_v4(smem_u32(smem) + (uint32_t)(i * 16), make_uint4(0u, 0u, 0u, 0u));
+  // zero the rows past each box once, and the input's tail: no copy writes them
+  // (a box is wi * nb rows of 128 bytes)
+  {
+    const int box = p.halo_wi * p.halo_ipr * 8;  // 16-byte pieces
+    for (int s = 0; s < Cfg::STAGES; ++s)
+      for (int b = 0; b < 3; ++b) {
+        const uint32_t base = smem_u32(smem + s * Cfg::STAGE + b * 16384);
+        const int end = b < 2 ? 16384 / 16 : Cfg::X_BYTES / 16;
+        for (int i = box + threadIdx.x; i < end; i += blockDim.x)
+          st_shared_v4(base + (uint32_t)(i * 16), make_uint4(0u, 0u, 0u, 0u));
+      }
+  }
   fence_proxy_async_smem();
   if (threadIdx.x == 0) {
     for (int s = 0; s < Cfg::STAGES; ++s) {
@@ -480,7 +493,7 @@ __global__ void __launch_bounds__(kWideWgradThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_u32(&tfull[a]), 1);
-      mbar_init(smem_u32(&tempty[a]), 4);
+      mbar_init(smem_u32(&tempty[a]), 8);
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -587,10 +600,11 @@ __global__ void __launch_bounds__(kWideWgradThreads, 1)
       if (!ok) record_timeout(p, abort_flag);
     }
   } else {
-    // epilogue warps 2..5: TMEM sub-partition warp % 4 holds output channels
+    // epilogue warps 2..9: TMEM sub-partition warp % 4 holds output channels
     // kt * 128 + 32 * (warp % 4) + lane; a lane writes its channel's three
-    // 64-wide runs (s = 0, 1, 2) of the unit's filter row
-    const int sub = warp & 3;
+    // 64-wide runs (s = 0, 1, 2) of the unit's filter row, the sub-partition's two
+    // warps 32 columns of each
+    const int sub = warp & 3, half = (warp - 2) >> 2;
     const int C = p.halo_chunks * 64;
     int acc = 0;
     uint32_t acc_phase = 0;
@@ -608,22 +622,20 @@ __global__ void __launch_bounds__(kWideWgradThreads, 1)
 #pragma unroll 1
       for (int s = 0; s < 3; ++s) {
         const uint32_t tb =
-            tmem_base + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * Cfg::ACC_COLS + s * 64);
-        uint32_t v[64];
+            tmem_base + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * Cfg::ACC_COLS + s * 64 + half * 32);
+        uint32_t v[32];
         tmem_ld16(tb, v);
         tmem_ld16(tb + 16, v + 16);
-        tmem_ld16(tb + 32, v + 32);
-        tmem_ld16(tb + 48, v + 48);
         tmem_ld_wait();
-        if (p.d_f32) f32_to_f16_lo<64>(v);  // FP32 accumulator: one rounding to FP16
+        if (p.d_f32) f32_to_f16_lo<32>(v);  // FP32 accumulator: one rounding to FP16
         if (s == 2) {  // accumulator fully read: hand it back before the stores
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&tempty[acc]));
         }
-        uint4* dst = reinterpret_cast<uint4*>(prow + (size_t)s * C);
+        uint4* dst = reinterpret_cast<uint4*>(prow + (size_t)s * C + half * 32);
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+        for (int j = 0; j < 4; ++j)
           dst[j] = make_uint4(pack_lo(v[j * 8 + 0], v[j * 8 + 1]), pack_lo(v[j * 8 + 2], v[j * 8 + 3]),
                               pack_lo(v[j * 8 + 4], v[j * 8 + 5]), pack_lo(v[j * 8 + 6], v[j * 8 + 7]));
       }
