@@ -570,6 +570,12 @@ constexpr int kStatRowsT = 8;                   // rows per consumer thread per 
 constexpr int kStatStages = 3;                  // shared-memory ring depth
 constexpr int kStatLevels = 9;                  // per-thread chunk trees: up to 256 chunks
 constexpr int kStatMaxChunks = 1 << (kStatLevels - 1);
+// levels of the backward's chunk trees kept in registers: most tensors leave a CTA
+// at most eight chunks, and the indexed stack above them is local memory (its
+// loads were the statistics' first stall; 28x28x512 at batch 64 backward 54.7 ->
+// 53.8 us, 112x112x64 at batch 256 311 -> 307 us; the forward, whose nodes are
+// larger and whose CTAs share the SM, got slower with it)
+constexpr int kRegLevels = 3;
 constexpr int kStatTensorBytes = kStatRowsT * kBnThreads * 16;  // one tensor's slot: RB rows <= 32 KB
 constexpr int kFwdCtasPerSm = 2;                // forward ring: 3 x 32 KB (x)
 constexpr int kBwdCtasPerSm = 1;                // backward ring: 3 x 64 KB (x, dy)
@@ -881,7 +887,7 @@ __global__ void __launch_bounds__(kBnThreads + 32, kBwdCtasPerSm) k_bn_bwd_stats
     }
   };
   if (RELU != BN_NO_RELU) load_relu(0);
-  uint4 st1[kStatLevels], st2[kStatLevels];
+  uint4 rt1[kRegLevels], rt2[kRegLevels], st1[kStatLevels - kRegLevels], st2[kStatLevels - kRegLevels];
   unsigned cnt = 0;
   bool ok = true;
   for (int ci = 0;; ++ci) {
@@ -921,15 +927,29 @@ __global__ void __launch_bounds__(kBnThreads + 32, kBwdCtasPerSm) k_bn_bwd_stats
     __syncwarp();
     if ((t & 31) == 0) mbar_arrive(bars + 8 * (kStatStages + s));
     uint4 n1 = sum8(p1), n2 = sum8(p2);
+    bool carry = true;
+#pragma unroll
+    for (int l = 0; l < kRegLevels; ++l) {
+      if (carry && (cnt >> l & 1u)) {
+        n1 = add4(rt1[l], n1);
+        n2 = add4(rt2[l], n2);
+      } else if (carry) {
+        rt1[l] = n1;
+        rt2[l] = n2;
+        carry = false;
+      }
+    }
+    if (carry) {
 #pragma unroll 1
-    for (int l = 0; l < kStatLevels; ++l) {
-      if (cnt & (1u << l)) {
-        n1 = add4(st1[l], n1);
-        n2 = add4(st2[l], n2);
-      } else {
-        st1[l] = n1;
-        st2[l] = n2;
-        break;
+      for (int l = kRegLevels; l < kStatLevels; ++l) {
+        if (cnt & (1u << l)) {
+          n1 = add4(st1[l - kRegLevels], n1);
+          n2 = add4(st2[l - kRegLevels], n2);
+        } else {
+          st1[l - kRegLevels] = n1;
+          st2[l - kRegLevels] = n2;
+          break;
+        }
       }
     }
     ++cnt;
@@ -938,22 +958,25 @@ __global__ void __launch_bounds__(kBnThreads + 32, kBwdCtasPerSm) k_bn_bwd_stats
   // close the chunk trees as if zero chunks padded them to 2^chunk_levels
   uint4 acc1 = zero4(), acc2 = zero4();
   bool have = false;
-#pragma unroll 1
-  for (int l = 0; l < kStatLevels; ++l) {
+  auto close = [&](int l, const uint4& v1, const uint4& v2) {
     if (l < a.chunk_levels) {
       if (cnt & (1u << l)) {
-        acc1 = add4(st1[l], have ? acc1 : zero4());
-        acc2 = add4(st2[l], have ? acc2 : zero4());
+        acc1 = add4(v1, have ? acc1 : zero4());
+        acc2 = add4(v2, have ? acc2 : zero4());
         have = true;
       } else if (have) {
         acc1 = add4(acc1, zero4());
         acc2 = add4(acc2, zero4());
       }
     } else if (l == a.chunk_levels && (cnt & (1u << l))) {
-      acc1 = st1[l];
-      acc2 = st2[l];
+      acc1 = v1;
+      acc2 = v2;
     }
-  }
+  };
+#pragma unroll
+  for (int l = 0; l < kRegLevels; ++l) close(l, rt1[l], rt2[l]);
+#pragma unroll 1
+  for (int l = kRegLevels; l < kStatLevels; ++l) close(l, st1[l - kRegLevels], st2[l - kRegLevels]);
   s1[t] = acc1;
   s2[t] = acc2;
   consumers_sync(ncons);
