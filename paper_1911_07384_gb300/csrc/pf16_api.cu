@@ -186,13 +186,30 @@ int pick_bn_out(long long n) {  // tile width for an output of n columns
 // K-block from ~500 to ~270 (128) and ~180 (64) cycles of MMA and half of its
 // weight traffic off that chain.  The classifier's forward at batch 256 (8
 // tiles of 256, 32 K-blocks each): 22.4 -> 18.4 us with 32 tiles of 64, its
-// data gradient 16.3 -> 12.3 us.  The rule stops where the tiles would outnumber the SMs (a second round costs
-// more than it saves), so a fused-statistics launch keeps one tile, hence one
-// slot, per M tile and the same statistics tree.
+// data gradient 16.3 -> 12.3 us.  The rule stops where the tiles would
+// outnumber the SMs (a second round costs more than it saves), so a
+// fused-statistics launch keeps one tile, hence one slot, per M tile and the
+// same statistics tree.
 int fill_bn(int bn, long long m_tiles, long long n, int sms) {
   for (int half : {128, 64})
     if (half < bn && m_tiles * ((n + half - 1) / half) <= sms) bn = half;
   return bn;
+}
+// The same, and 128 columns in place of 256 where the last round of 256-wide
+// tiles would leave so many SMs idle that the narrower tiles' rounds, each 0.56
+// as long (shared-memory bandwidth keeps it above half), end sooner.  98 x 2
+// tiles of 256 are two rounds, 98 x 4 of 128 three: at batch 256 the 7 x 7
+// 512 -> 512 3x3 forward 48.8 -> 44.9 us and data gradient 48.4 -> 43.6, the
+// 1x1 2048 -> 512 forward 28.8 -> 25.6; the four phases of the strided 3x3's data
+// gradient into 14 x 14 x 512 at batch 64 17.8 -> 16.2; 28 x 28 512 -> 320 at
+// batch 64 25.4 -> 22.7.  392 x 1 tiles (2.6 rounds) stay at 256: 49.6 us against
+// 53.7 (14 x 14 256 -> 256 with backward statistics).  Not for launches with
+// statistics, whose trees follow the tiles.
+int round_bn(int bn, long long m_tiles, long long n, int sms) {
+  bn = fill_bn(bn, m_tiles, n, sms);
+  if (bn != 256) return bn;
+  auto rounds = [&](int w) { return (m_tiles * ((n + w - 1) / w) + sms - 1) / sms; };
+  return 56 * rounds(128) < 100 * rounds(256) ? 128 : 256;
 }
 int pick_bn_wgrad(long long n) {
   if (n % 256 == 0) return 256;
@@ -576,7 +593,7 @@ int run_dgrad_phases(const Shape& s, const uint16_t* dy, const uint16_t* w, uint
   CUtensorMap ma, mb;
   p.M = (int)(s.N * gh * gw);
   p.N = (int)s.C;
-  BN = fill_bn(BN, 4ll * cdiv(p.M, kBM), s.C, sms);
+  BN = (stats ? fill_bn : round_bn)(BN, 4ll * cdiv(p.M, kBM), s.C, sms);
   p.a_mode = LD_IM2COL_K;
   p.b_mode = LD_TAP3D_MN;
   set_kmajor(p, true, false);
@@ -917,7 +934,7 @@ static int conv_fwd_impl(const pf16_conv_desc* d, const uint16_t* x, const uint1
   if (const int ws_s2d = stem_s2d_width(s, (flags & PF16_ACCUMULATE) != 0))
     return run_stem_s2d(s, ws_s2d, x, w, y, ws, status, sms, st, stats, f32);
   set_stats(p, stats, s.K);
-  const int BN = fill_bn(pick_bn_out(s.K), cdiv(p.M, kBM), s.K, sms);
+  const int BN = (stats ? fill_bn : round_bn)(pick_bn_out(s.K), cdiv(p.M, kBM), s.K, sms);
   p.a_mode = LD_TILED_K;
   p.b_mode = LD_TILED_K;
   set_kmajor(p, true, true);
@@ -1033,7 +1050,7 @@ static int conv_dgrad_impl(const pf16_conv_desc* d, const uint16_t* dy, const ui
     CUtensorMap ma, mb;
     p.M = (int)(s.N * s.P * s.Q);
     p.N = (int)s.C;
-    const int BN = fill_bn(bn_max, cdiv(p.M, kBM), s.C, sms);
+    const int BN = (stats ? fill_bn : round_bn)(bn_max, cdiv(p.M, kBM), s.C, sms);
     p.a_mode = LD_TILED_K;
     p.b_mode = LD_TILED_MN;
     set_kmajor(p, true, false);
@@ -1079,7 +1096,7 @@ static int conv_dgrad_impl(const pf16_conv_desc* d, const uint16_t* dy, const ui
       CUtensorMap ma, mb;
       p.M = (int)(s.N * gh * gw);
       p.N = (int)s.C;
-      const int BN = fill_bn(bn_max, cdiv(p.M, kBM), s.C, sms);
+      const int BN = (stats ? fill_bn : round_bn)(bn_max, cdiv(p.M, kBM), s.C, sms);
       p.a_mode = LD_IM2COL_K;
       p.b_mode = LD_TAP3D_MN;
       set_kmajor(p, true, false);

@@ -192,9 +192,12 @@ __host__ __device__ inline size_t bnstat_bytes(long long C) {
 // take the TMA-fed epilogue for short reductions (at most kTmaEpiMaxKb
 // K-blocks per tile: there the epilogue's traffic is the bound) and always
 // with an addend; else their inputs go through registers, which leaves the
-// main loop all of its pipeline stages.
+// main loop all of its pipeline stages.  TMA-fed against registers at 28 x 28,
+// batch 64, dx of 512 (320 for the first): four K-blocks 30.5 / 33.4 us, five
+// 38.5 / 37.4, six 42.1 / 38.7, eight (dx of 128) 19.3 / 18.0; at batch 256 four
+// (14 x 14 256 -> 1024) 57.9 / 68.2, eight (7 x 7 512 -> 2048) 45.8 / 41.1.
 enum GemmEpi : int { EPI_PLAIN = 0, EPI_BS = 1, EPI_BS_TMA = 2, EPI_BS_ADD = 3, EPI_BS_REMAP = 4 };
-constexpr int kTmaEpiMaxKb = 8;
+constexpr int kTmaEpiMaxKb = 4;
 inline int gemm_epilogue(const GemmParams& p) {
   if (!p.bs_x) return EPI_PLAIN;
   if (p.add_src) return EPI_BS_ADD;
