@@ -1035,20 +1035,25 @@ cudaError_t launch_gemm(int BN, const CUtensorMap& mA, const CUtensorMap& mB, co
 // TMA store, which clips at Q.
 // Same roles and bounded waits as k_gemm.
 // ---------------------------------------------------------------------------
+// SW: the stem with statistics warps (k_gemm_halo)
+template <bool SW>
 struct HaloCfg {
-  static constexpr int B_BYTES = 9 * 64 * kBK * 2;  // resident: 9 taps x 64 x 64, or 16 x 64 x 16
-  static constexpr int A_BOX_MAX = 64 * 4 * 128;    // ws = 64: 4 rows of 64 pixels (ws = 32: 6 x 32;
-                                                    // the stem: 4 rows of 128 pixels x 32 bytes)
+  static constexpr int B_BYTES = SW ? 16 * 64 * 32 : 9 * 64 * kBK * 2;  // resident: 9 taps x 64 x 64, or 16 x 64 x 16
+  static constexpr int A_BOX_MAX = SW ? 4 * 128 * 32       // the stem: 4 rows of 128 pixels x 32 bytes
+                                      : 64 * 4 * 128;      // ws = 64: 4 rows of 64 pixels (ws = 32: 6 x 32)
   static constexpr int A_STAGE = A_BOX_MAX + 1024;  // + the last tap window's over-read (the stem)
-  static constexpr int STAGES = 3;
-  static constexpr int STAGING_BYTES = kEpiWarps * 4096;  // one 32 x 64 tile per epilogue warp
+  static constexpr int STAGES = SW ? 6 : 3;
+  static constexpr int STAGING_BYTES = kEpiWarps * (SW ? 2 : 1) * 4096;  // 32 x 64 tiles of the epilogue warps
   // 3x3: rows 0 and 1 of each warp's shifted partials (128 32-bit columns),
-  // per epilogue group, tile parity and TMEM sub-partition
-  static constexpr int XCH_BYTES = 2 * 2 * 4 * 2 * 512;
-  static constexpr int BAR_BYTES = 8 * (2 * STAGES + 7) + 16;
+  // per epilogue group, tile parity and TMEM sub-partition.  SW: the
+  // statistics' closing merge.
+  static constexpr int XCH_BYTES = SW ? 9 * 1024 : 2 * 2 * 4 * 2 * 512;
+  static constexpr int SBARS = SW ? 2 * 2 * kEpiWarps : 0;  // staging tiles' full and empty barriers
+  static constexpr int BAR_BYTES = 8 * (2 * STAGES + 7 + SBARS) + 16;
   static constexpr int SMEM = 1024 + B_BYTES + STAGES * A_STAGE + STAGING_BYTES + XCH_BYTES + BAR_BYTES;
   static_assert(SMEM <= 232448, "shared memory per CTA");
 };
+constexpr int kHaloThreadsSw = kGemmThreads + 32 * kEpiWarps;
 
 // 3x3 halo epilogue.  The accumulator holds in columns 64 j + c (j = 0, 1, 2)
 // the products of taps (r, j) read through the window of tap (r, 0), summed
@@ -1129,11 +1134,22 @@ __device__ __forceinline__ void halo3_combine(uint32_t tb, int lane, bool f32, b
 // start-address field is the low 14 bits; desc_addr16 masks a shared address
 // into it, and a stage plus its tap offsets stays below 256 KB), so a single
 // thread keeps up with N = 64 MMAs.
-template <int CB, bool BS>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+//
+// SW (the stem's forward over many tiles): two staging tiles per epilogue warp,
+// so that a drain never waits for the previous tile's store, and the statistics
+// taken from them by eight more warps.  In one chain, drain and statistics of a
+// tile took ~2,400 cycles of its epilogue group, above twice the ~1,000 cycles
+// of its MMAs.  Batch 128 of the 224 x 224 stem, with the space-to-depth pass's
+// 19 us: with statistics 93.0 -> 82.3 us, without 81.2 -> 71.8; 32 x 160 x 160
+// with statistics 22.5 -> 21.0.  Statistics warp e takes epilogue warp e's tiles
+// in their order, so the trees are the same.  What bounds it now is the MMAs
+// (~62 cycles each at N = 64) and the output's stores, ~50 us each.
+template <int CB, bool BS, bool SW>
+__global__ void __launch_bounds__(SW ? kHaloThreadsSw : kGemmThreads, 1)
     k_gemm_halo(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ CUtensorMap mapC, const __grid_constant__ GemmParams p) {
-  using Cfg = HaloCfg;
+  using Cfg = HaloCfg<SW>;
+  static_assert(!SW || (CB == 32 && !BS), "statistics warps: the stem's forward");
   constexpr int NTAPS = CB == 128 ? 9 : 16;
   constexpr int KSTEPS = CB / 32;                 // K = 16 steps per tap
   constexpr uint32_t SWZ = CB == 128 ? 2u : 6u;   // descriptor swizzle code
@@ -1154,7 +1170,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   uint64_t* tempty = tfull + 2;
   uint64_t* bready = tempty + 2;
   uint64_t* xbar = bready + 1;  // per epilogue group: the exchange of shifted partials
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(xbar + 2);
+  uint64_t* sfull = xbar + 2;  // [kEpiWarps][2]: staging tiles written, and read by their statistics warp
+  uint64_t* sempty = sfull + Cfg::SBARS / 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(xbar + 2 + Cfg::SBARS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int ws = p.halo_ws, rows = kBM / ws;
@@ -1176,6 +1194,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     tma_prefetch_desc(&mapA);
     tma_prefetch_desc(&mapB);
     tma_prefetch_desc(&mapC);
+  }
+  if (SW && warp == 2) {
+    static_assert(!SW || Cfg::SBARS == 32, "a barrier per lane");
+    mbar_init(smem_u32(&sfull[lane]), 1);
+    fence_mbar_init();
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
@@ -1288,6 +1311,33 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if (acc == 0) acc_phase ^= 1;
       }
     }
+  } else if (SW && warp >= 2 + kEpiWarps) {
+    // statistics warps 10..17 (launched when there are statistics): warp e takes
+    // the tiles that epilogue warp e stages, in its order
+    const int e = warp - 2 - kEpiWarps, grp = e >> 2, sub = (e + 2) & 3;
+    EpiStats stats;
+    stats.init();
+    uint32_t it = 0;
+    for (int u = blockIdx.x + grp * gridDim.x; u < total; u += 2 * gridDim.x, ++it) {
+      const int b = e * 2 + (int)(it & 1);
+      const bool got = mbar_wait(smem_u32(&sfull[b]), (it >> 1) & 1, lim);
+      if (!__all_sync(0xffffffffu, got && *abort_flag == 0)) {
+        if (lane == 0 && !got) record_timeout(p, abort_flag);
+        break;
+      }
+      const int nv = min(32, max(0, p.halo_w - (u * kBM + sub * 32) % ws));  // columns j >= W are padding
+      if (nv > 0) {
+        stats.leaf(0, smem_u32(staging) + (uint32_t)(b * 4096), lane, nv);
+        stats.end_tile(nv);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sempty[b]));
+    }
+    stats.write_cta(p, xch, e, blockIdx.x, 0, 1, lane, true);
+    if (blockIdx.x == 0 && e == 0 && lane == 0) {
+      p.st_hdr[0] = (int)gridDim.x;
+      p.st_hdr[1] = 5 + p.bs_levels + 3;
+    }
   } else {
     // epilogue warps 2..9: group (w - 2) / 4 drains accumulator 0 or 1 (the
     // CTA's even or odd tiles), warp w its TMEM sub-partition w % 4; 32 rows
@@ -1295,7 +1345,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int e = warp - 2, grp = e >> 2, sub = warp & 3;
     const int acc = grp;
     uint32_t acc_phase = 0;
-    const uint32_t stg = smem_u32(staging) + (uint32_t)(e * 4096);
+    uint32_t stg = smem_u32(staging) + (uint32_t)(e * (SW ? 8192 : 4096));
+    uint32_t it = 0;  // tiles staged
     EpiStats stats;
     stats.init();
     BwdIn bin;
@@ -1350,7 +1401,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&tempty[acc]));
-      if (lane == 0) bulk_wait_read0();  // the previous store has read the staging tile
+      if constexpr (SW) {  // the buffer's store and statistics, two tiles back, have read it
+        stg = smem_u32(staging) + (uint32_t)((e * 2 + (int)(it & 1)) * 4096);
+        const bool free = !p.st_mean || mbar_wait(smem_u32(&sempty[e * 2 + (it & 1)]), ((it >> 1) & 1) ^ 1, lim);
+        if (!__all_sync(0xffffffffu, free)) {
+          if (lane == 0) record_timeout(p, abort_flag);
+          break;
+        }
+        if (lane == 0) bulk_wait_read1();
+      } else {
+        if (lane == 0) bulk_wait_read0();  // the previous store has read the staging tile
+      }
       __syncwarp();
 #pragma unroll
       for (int j = 0; j < 8; ++j)
@@ -1363,10 +1424,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const int grow = mp / ws, col = mp - grow * ws;
         if (col < p.halo_w) {  // a box wholly right of the image has nothing to store
           tma_store_3d(&mapC, stg, 0, col, grow);
+          if (!SW) bulk_commit();
+        }
+        if (SW) {  // (one group a tile, an empty one too)
           bulk_commit();
+          if (p.st_mean) mbar_arrive(smem_u32(&sfull[e * 2 + (it & 1)]));
         }
       }
-      if (p.st_mean) {
+      ++it;
+      if (!SW && p.st_mean) {
         const int mp = u * kBM + sub * 32;
         const int nv = min(32, max(0, p.halo_w - mp % ws));  // columns j >= W are padding
         if (nv > 0) {
@@ -1380,7 +1446,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       acc_phase ^= 1;
     }
     if (lane == 0) bulk_wait0();
-    if (p.st_mean) {
+    if (!SW && p.st_mean) {
       if (BS)
         stats.write_cta_bwd(p, staging, e, blockIdx.x, 0, 1, lane, p.bs_levels);
       else
@@ -1407,10 +1473,19 @@ cudaError_t launch_gemm_halo(const CUtensorMap& mA, const CUtensorMap& mB, const
     for (int t = 0; t < p.ntaps; ++t) m = max(m, (p.tap_dr[t] * p.halo_ws + p.tap_ds[t]) * p.halo_cb);
     return m;
   }();
+  // Statistics warps and double staging from eight tiles a CTA on, double
+  // staging alone (no statistics) from 32: with fewer the longer set-up costs
+  // more (with statistics 1.3 tiles: 8.3 -> 8.6 us, 5.9: 12.7 -> 13.0, 17: 23.8 ->
+  // 22.3, 67: 66.9 -> 59.6; without 17: 18.9 -> 19.3, 67: 53.8 -> 52.3).
+  const bool sw = p.halo_cb == 32 && p.m_tiles >= (p.st_mean ? 8 : 32) * grid;
+  auto too_big = [&](int b, int box, int stage) {
+    return p.ntaps * 64 * p.halo_cb > b || p.halo_box_rows * p.halo_ws * p.halo_cb > box ||
+           max_off + kBM * p.halo_cb > stage;
+  };
   if (p.ntaps != (p.halo_cb == 128 ? 9 : 16) || (p.halo_cb != 128 && p.halo_cb != 32) || p.halo_ws <= 0 ||
-      kBM % p.halo_ws != 0 || p.ntaps * 64 * p.halo_cb > HaloCfg::B_BYTES ||
-      p.halo_box_rows * p.halo_ws * p.halo_cb > HaloCfg::A_BOX_MAX ||
-      max_off + kBM * p.halo_cb > HaloCfg::A_STAGE)
+      kBM % p.halo_ws != 0 ||
+      (sw ? too_big(HaloCfg<true>::B_BYTES, HaloCfg<true>::A_BOX_MAX, HaloCfg<true>::A_STAGE)
+          : too_big(HaloCfg<false>::B_BYTES, HaloCfg<false>::A_BOX_MAX, HaloCfg<false>::A_STAGE)))
     return cudaErrorInvalidValue;
   // 3x3: slot t holds tap (t / 3, t % 3), so filter row r's three slices are
   // the contiguous N = 192 operand read through tap (r, 0)'s window
@@ -1418,19 +1493,22 @@ cudaError_t launch_gemm_halo(const CUtensorMap& mA, const CUtensorMap& mB, const
     for (int t = 0; t < 9; ++t)
       if (p.tap_dr[t] != t / 3 || p.tap_ds[t] != t % 3) return cudaErrorInvalidValue;
   // variants: 128-byte pixels, with backward statistics (the 3x3 data gradient) or not; 32-byte pixels
-  static bool attr_set[3][64] = {};
+  static bool attr_set[4][64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
-  const int v = p.halo_cb == 128 ? (p.bs_x ? 1 : 0) : 2;
-  if (v == 2 && p.bs_x) return cudaErrorInvalidValue;
-  void (*const kern[3])(CUtensorMap, CUtensorMap, CUtensorMap, GemmParams) = {
-      k_gemm_halo<128, false>, k_gemm_halo<128, true>, k_gemm_halo<32, false>};
+  const int v = p.halo_cb == 128 ? (p.bs_x ? 1 : 0) : (sw ? 3 : 2);
+  if (v >= 2 && p.bs_x) return cudaErrorInvalidValue;
+  void (*const kern[4])(CUtensorMap, CUtensorMap, CUtensorMap, GemmParams) = {
+      k_gemm_halo<128, false, false>, k_gemm_halo<128, true, false>, k_gemm_halo<32, false, false>,
+      k_gemm_halo<32, false, true>};
+  const int smem = sw ? HaloCfg<true>::SMEM : HaloCfg<false>::SMEM;
   if (dev < 64 && !attr_set[v][dev]) {
-    cudaError_t e = cudaFuncSetAttribute(kern[v], cudaFuncAttributeMaxDynamicSharedMemorySize, HaloCfg::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(kern[v], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     attr_set[v][dev] = true;
   }
-  launch_pdl(kern[v], dim3(grid), dim3(kGemmThreads), HaloCfg::SMEM, s, mA, mB, mC, p);
+  const int threads = sw && p.st_mean ? kHaloThreadsSw : kGemmThreads;
+  launch_pdl(kern[v], dim3(grid), dim3(threads), (size_t)smem, s, mA, mB, mC, p);
   return counted_launches(1);
 }
 
