@@ -1187,7 +1187,7 @@ static int run_stem_wgrad(const Shape& s, const StemWgradPlan& sw, const uint16_
   {
     cuuint64_t dims[4] = {16, (cuuint64_t)Wsd, (cuuint64_t)Hs, (cuuint64_t)N};
     cuuint64_t strides[3] = {32, (cuuint64_t)(Wsd * 32), (cuuint64_t)(Hs * Wsd * 32)};
-    cuuint32_t box[4] = {16, 128, 4, 1};
+    cuuint32_t box[4] = {16, 128, 1, 1};
     if (g_encode_tiled(&mxs, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, xs, dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)

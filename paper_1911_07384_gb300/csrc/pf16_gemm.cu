@@ -1527,8 +1527,11 @@ cudaError_t launch_gemm_halo(const CUtensorMap& mA, const CUtensorMap& mB, const
 // (u + 1, v) over output row i - 1; u = 0 and u = 2 cover all sixteen taps
 // when i runs over 0..P (dy rows -1 and P read as zeros).  A work unit is
 // one (image, i) row: a stage holds dy rows i - 1, i (2 x 128 x 128 B) and
-// xs rows i .. i + 3 (4 x 128 x 32 B; windows reach at most 3 pixels into
-// row i + 3, and only at padding columns, where dy is zero).  Units are
+// xs rows i and i + 2 (128 x 32 B each, then a gap that stays zero: windows
+// reach at most 3 pixels past 128 columns, where dy is zero too).  With rows
+// i + 1 and i + 3 loaded as well, which only those 3 pixels reached, tiled TMA's
+// 32-byte rows took 50 us of the kernel at batch 128 of the 224 x 224 stem, and a
+// stage less fitted: 81.6 -> 77.3 us for the call.  Units are
 // accumulated in FP16 in TMEM over chunks of p.kb_per_split rows (4,096
 // padded pixels at ws = 128), and each chunk's 128 x 128 FP16 partial
 // [(a, k)][(u/2, v, ch)] goes to p.out + chunk * 128 * 128 for the split-K
@@ -1537,9 +1540,10 @@ cudaError_t launch_gemm_halo(const CUtensorMap& mA, const CUtensorMap& mB, const
 struct StemWgradCfg {
   static constexpr int WS = 128;
   static constexpr int DY_BYTES = 2 * WS * 128;   // dy rows i - 1, i
-  static constexpr int XS_BYTES = 4 * WS * 32;    // xs rows i .. i + 3
+  static constexpr int XS_SLOT = WS * 32 + 512;
+  static constexpr int XS_BYTES = 2 * XS_SLOT;    // xs rows i, i + 2
   static constexpr int STAGE = DY_BYTES + XS_BYTES;
-  static constexpr int STAGES = 4;
+  static constexpr int STAGES = 5;
   static constexpr int TMEM_COLS = 256;           // two 128-column accumulators
   static constexpr int BAR_BYTES = 8 * (2 * STAGES + 4) + 16;
   static constexpr int SMEM = 1024 + STAGES * STAGE + BAR_BYTES;
@@ -1576,6 +1580,12 @@ __global__ void __launch_bounds__(kStemWgradThreads, 1)
     tma_prefetch_desc(&mapDy);
     tma_prefetch_desc(&mapXs);
   }
+  if (warp >= 2) {  // the gaps: 512 bytes a slot
+    for (int z = warp - 2; z < 2 * Cfg::STAGES; z += 4)
+      *reinterpret_cast<uint4*>(smem + (z >> 1) * Cfg::STAGE + Cfg::DY_BYTES + (z & 1) * Cfg::XS_SLOT + Cfg::WS * 32 +
+                                lane * 16) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
+  }
   if (warp == 1) {
     tmem_alloc(smem_u32(tmem_slot), Cfg::TMEM_COLS);
     tmem_relinquish();
@@ -1605,9 +1615,10 @@ __global__ void __launch_bounds__(kStemWgradThreads, 1)
           }
           const uint32_t fb = smem_u32(&full[stage]);
           const uint32_t dst = smem_u32(smem + stage * Cfg::STAGE);
-          mbar_arrive_expect_tx(fb, (uint32_t)Cfg::STAGE);
+          mbar_arrive_expect_tx(fb, (uint32_t)(Cfg::DY_BYTES + 2 * Cfg::WS * 32));
           tma_load_4d(dst, &mapDy, fb, 0, 0, i - 1, n);
           tma_load_4d(dst + Cfg::DY_BYTES, &mapXs, fb, 0, 0, i, n);
+          tma_load_4d(dst + Cfg::DY_BYTES + Cfg::XS_SLOT, &mapXs, fb, 0, 0, i + 2, n);
           ++issued;
           if (++stage == Cfg::STAGES) {
             stage = 0;
@@ -1663,7 +1674,7 @@ __global__ void __launch_bounds__(kStemWgradThreads, 1)
 #pragma unroll
             for (int uu = 0; uu < 2; ++uu)
               tc_mma_f16(d_tmem + (uint32_t)(uu * 64), ab + (uint32_t)(js * (2048 >> 4)),
-                         bb + (uint32_t)((uu * 2 * Cfg::WS * 32 + js * 512) >> 4), p.idesc,
+                         bb + (uint32_t)((uu * Cfg::XS_SLOT + js * 512) >> 4), p.idesc,
                          (g > g0 || js > 0) ? 1u : 0u);
           tc_commit(smem_u32(&empty[stage]));
           if (++stage == Cfg::STAGES) {
