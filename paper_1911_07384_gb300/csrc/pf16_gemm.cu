@@ -778,6 +778,14 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
         const int nv0 = min(32, max(0, p.M - (m0 + sub * 32)));
         if (nv0 > 0) bin.load(p, (long long)(m0 + sub * 32), n0, nv0, lane);
       }
+      // remapped rows: lane l finds row l's place while the accumulator is computed
+      // (eight rows a lane, after the wait, put ~24 integer divisions into every
+      // drain: batch 64, 56 x 56 128-128 stride-2 3x3 26.0 -> 21.1 us)
+      unsigned long long place = 0;
+      if (!XF && !p.tma_store) {
+        const int m = m0 + sub * 32 + lane;
+        if (m < p.M) place = reinterpret_cast<unsigned long long>(out_row(p, m, split));
+      }
       const bool got = mbar_wait(smem_u32(&tfull[acc]), acc_phase, lim);
       if (!__all_sync(0xffffffffu, got)) {
         if (lane == 0) record_timeout(p, abort_flag);
@@ -846,10 +854,8 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
         const int rq = lane >> 3, cj = lane & 7;
         uint16_t* orow[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int m = m0 + sub * 32 + rq + 4 * i;
-          orow[i] = m < p.M ? out_row(p, m, split) : nullptr;
-        }
+        for (int i = 0; i < 8; ++i)
+          orow[i] = reinterpret_cast<uint16_t*>(__shfl_sync(0xffffffffu, place, rq + 4 * i));
 #pragma unroll 1
         for (int c = 0; c < BN; c += 64) {
           uint32_t r[64];
