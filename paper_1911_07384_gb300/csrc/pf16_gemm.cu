@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
       // (eight rows a lane, after the wait, put ~24 integer divisions into every
       // drain: batch 64, 56 x 56 128-128 stride-2 3x3 26.0 -> 21.1 us)
       unsigned long long place = 0;
-      if (!XF && !p.tma_store) {
+      if (!XF && !WE && !p.tma_store) {
         const int m = m0 + sub * 32 + lane;
         if (m < p.M) place = reinterpret_cast<unsigned long long>(out_row(p, m, split));
       }
@@ -793,7 +793,7 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
       }
       tc_fence_after();
       const uint32_t tbase = tmem_base + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * BN);
-      if (p.tma_store) {
+      if (WE || p.tma_store) {  // (the wide epilogue is only launched with TMA stores)
         // valid rows of this warp (a prefix of its 32) for the fused statistics
         const int nv = min(32, max(0, p.M - (m0 + sub * 32)));
         // 64-column chunks: TMEM -> registers -> 128B-swizzled staging -> TMA store
@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
         acc_phase ^= 1;
         continue;
       }
-      if constexpr (!XF) {  // (the operand-transform variants never take remapped rows)
+      if constexpr (!XF && !WE) {  // (the operand-transform variants never take remapped rows)
         // Rows remapped to strided positions (a stride phase): each 64-column
         // chunk goes through the warp's 128B-swizzled staging tile, then lane l
         // moves 16 bytes (columns 8 (l % 8) ..) of rows l / 8 + 4 i, i < 8: a
