@@ -1534,10 +1534,10 @@ cudaError_t launch_gemm_halo(const CUtensorMap& mA, const CUtensorMap& mB, const
 // when i runs over 0..P (dy rows -1 and P read as zeros).  A work unit is
 // one (image, i) row: a stage holds dy rows i - 1, i (2 x 128 x 128 B) and
 // xs rows i and i + 2 (128 x 32 B each, then a gap that stays zero: windows
-// reach at most 3 pixels past 128 columns, where dy is zero too).  With rows
-// i + 1 and i + 3 loaded as well, which only those 3 pixels reached, tiled TMA's
-// 32-byte rows took 50 us of the kernel at batch 128 of the 224 x 224 stem, and a
-// stage less fitted: 81.6 -> 77.3 us for the call.  Units are
+// reach at most 3 pixels past 128 columns, where dy is zero too).  Rows i + 1 and
+// i + 3, which only those 3 pixels reached, were loaded as well: without them the
+// call at batch 128 of the 224 x 224 stem goes 81.6 -> 79.2 us, and with the fifth
+// stage that then fits 77.3.  Units are
 // accumulated in FP16 in TMEM over chunks of p.kb_per_split rows (4,096
 // padded pixels at ws = 128), and each chunk's 128 x 128 FP16 partial
 // [(a, k)][(u/2, v, ch)] goes to p.out + chunk * 128 * 128 for the split-K
