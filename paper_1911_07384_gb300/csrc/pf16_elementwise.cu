@@ -11,6 +11,7 @@
 
 #include "../../include/pf16.h"
 #include "pf16_internal.h"
+#include "pf16_plan.h"
 #include "pf16_ptx.cuh"
 
 namespace pf16 {
@@ -231,14 +232,15 @@ cudaError_t launch_dp_combine(const uint16_t* planes, int world, size_t n, size_
 }
 
 // ============================================================================
-// Split-K weight-gradient reduction: out = balanced pairwise FP16 tree over
-// the `splits` partial matrices.
+// Split-K weight-gradient reduction: out = the FP16 tree over the `splits`
+// partial matrices (pf16_plan.h states it).
 // ============================================================================
-// A CTA of 256 threads = cl output chunks (8 columns each) x grp split groups
-// (both powers of two); each thread sums an aligned run of NB <= 16 splits (zero
-// past the last one) as a perfect pairwise tree, all its loads in flight; then
-// the groups are summed pairwise in shared memory.  Every choice of grp sums
-// the same balanced tree over the padded splits.
+// A CTA of 256 threads = cl output chunks (8 columns each) x 2^groups_log2
+// groups of splits; each thread sums its NB <= 16 splits (zero past the last one)
+// as a perfect pairwise tree, all its loads in flight; then the groups meet in
+// shared memory, thread t and t + half, half halving.  A thread's place holds its
+// run's index in the low bits (the runs' sums meet at a stride, last) and above
+// them, mirrored, the group's place in the run (neighbours meet first).
 //
 // Bound by latency: the partials (1 to 10 MB) lie in L2 and the whole kernel is
 // one round of loads per thread, so what counts is the instruction path around
@@ -249,35 +251,45 @@ cudaError_t launch_dp_combine(const uint16_t* planes, int world, size_t n, size_
 // less; over 24 layers the weight gradients went from 921 to 819 us.
 template <int NB, bool DENSE>
 __global__ void __launch_bounds__(256)
-    k_splitk_reduce(const uint16_t* __restrict__ parts, int splits, int grp_log2, int total, int cpr, int plane,
-                    uint16_t* __restrict__ out, long long ldo, int cols_out) {
+    k_splitk_reduce(const uint16_t* __restrict__ parts, int splits, const SplitkPlan sk, int total, int cpr,
+                    int plane, uint16_t* __restrict__ out, long long ldo, int cols_out) {
   pdl_wait();
   __shared__ uint4 sh[256];
-  const int t = threadIdx.x, cl_log2 = 8 - grp_log2;
-  const int lane = t & ((1 << cl_log2) - 1), g = t >> cl_log2;
+  const int t = threadIdx.x, cl_log2 = 8 - sk.groups_log2;
+  const int lane = t & ((1 << cl_log2) - 1), tg = t >> cl_log2;
   const int chunk = (blockIdx.x << cl_log2) + lane;
   uint4 acc = zero4();
   if (chunk < total) {
-    const int first = g * NB;
-    const uint4* src = reinterpret_cast<const uint4*>(parts) + chunk + (long long)first * plane;
+    int first = tg;
+    if (NB != 2 || sk.leaf_step == 1) {
+      const int runs_log2 = min(sk.tree_groups_log2, sk.groups_log2), in_run = sk.groups_log2 - runs_log2;
+      const int run = tg & ((1 << runs_log2) - 1);
+      const int place = (int)(__brev((unsigned)(tg >> runs_log2)) >> ((32 - in_run) & 31));
+      first = ((run << in_run) + place) * NB;
+    }
+    const int step = NB == 2 ? sk.leaf_step : 1;
+    const uint4* src = reinterpret_cast<const uint4*>(parts) + chunk;
     uint4 v[NB];
 #pragma unroll
-    for (int i = 0; i < NB; ++i) v[i] = first + i < splits ? __ldg(src + (long long)i * plane) : zero4();
+    for (int i = 0; i < NB; ++i) {
+      const int sp = first + i * step;
+      v[i] = sp < splits ? __ldg(src + (long long)sp * plane) : zero4();
+    }
 #pragma unroll
     for (int w = 1; w < NB; w *= 2)
 #pragma unroll
       for (int i = 0; i + w < NB; i += 2 * w) v[i] = add4(v[i], v[i + w]);
     acc = v[0];
   }
-  if (grp_log2 > 0) {  // neighbouring groups' sums, pairwise
+  if (sk.groups_log2 > 0) {
     sh[t] = acc;
     __syncthreads();
-    for (int h = 1; h < (1 << grp_log2); h *= 2) {
-      if ((g & (2 * h - 1)) == 0) sh[t] = acc = add4(acc, sh[t + (h << cl_log2)]);
+    for (int half = 128; half >= (1 << cl_log2); half /= 2) {  // threads of half the groups
+      if (t < half) sh[t] = acc = add4(acc, sh[t + half]);
       __syncthreads();
     }
   }
-  if (g != 0 || chunk >= total) return;
+  if (tg != 0 || chunk >= total) return;
   if (DENSE) {
     reinterpret_cast<uint4*>(out)[chunk] = acc;
   } else {
@@ -292,35 +304,28 @@ __global__ void __launch_bounds__(256)
 
 template <int NB>
 static void launch_splitk_nb(bool dense, dim3 grid, cudaStream_t s, const uint16_t* parts, int splits,
-                             int grp_log2, int total, int cpr, int plane, uint16_t* out, long long ldo,
+                             const SplitkPlan& sk, int total, int cpr, int plane, uint16_t* out, long long ldo,
                              int cols_out) {
   launch_pdl(dense ? k_splitk_reduce<NB, true> : k_splitk_reduce<NB, false>, grid, dim3(256), 0, s, parts, splits,
-             grp_log2, total, cpr, plane, out, ldo, cols_out);
+             sk, total, cpr, plane, out, ldo, cols_out);
 }
 
 cudaError_t launch_splitk_reduce(const uint16_t* parts, int splits, long long rows, int cols,
                                  uint16_t* out, long long ldo, int cols_out, cudaStream_t s) {
-  int sp2 = 1;
-  while (sp2 < splits) sp2 *= 2;
   const long long total = rows * (cols / 8);  // 8-column chunks of the result
   if (total > (1ll << 30)) return cudaErrorInvalidValue;
   if (splits < 1 || splits > 4096) return cudaErrorInvalidValue;  // 256 groups of 16
-  // as many groups as leave a thread at most 16 splits, and more while the GPU
-  // has fewer than 512 threads per SM and a thread more than two loads (against
-  // 16 loads a thread throughout: 819 against 829 us over 24 weight gradients)
-  int grp_log2 = 0;
-  while ((sp2 >> grp_log2) > 16 || ((sp2 >> grp_log2) > 2 && (total << grp_log2) < 152ll * 512)) ++grp_log2;
-  const int seg = sp2 >> grp_log2;
-  const int cl = 256 >> grp_log2;
+  const SplitkPlan sk = splitk_plan(splits, total);
+  const int cl = 256 >> sk.groups_log2;
   const dim3 grid((unsigned)((total + cl - 1) / cl));
   const bool dense = ldo == cols && cols_out == cols && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
   const int cpr = cols / 8, plane = (int)total;
-  switch (seg) {
-    case 1: launch_splitk_nb<1>(dense, grid, s, parts, splits, grp_log2, (int)total, cpr, plane, out, ldo, cols_out); break;
-    case 2: launch_splitk_nb<2>(dense, grid, s, parts, splits, grp_log2, (int)total, cpr, plane, out, ldo, cols_out); break;
-    case 4: launch_splitk_nb<4>(dense, grid, s, parts, splits, grp_log2, (int)total, cpr, plane, out, ldo, cols_out); break;
-    case 8: launch_splitk_nb<8>(dense, grid, s, parts, splits, grp_log2, (int)total, cpr, plane, out, ldo, cols_out); break;
-    default: launch_splitk_nb<16>(dense, grid, s, parts, splits, grp_log2, (int)total, cpr, plane, out, ldo, cols_out); break;
+  switch (sk.leaves_log2) {
+    case 0: launch_splitk_nb<1>(dense, grid, s, parts, splits, sk, (int)total, cpr, plane, out, ldo, cols_out); break;
+    case 1: launch_splitk_nb<2>(dense, grid, s, parts, splits, sk, (int)total, cpr, plane, out, ldo, cols_out); break;
+    case 2: launch_splitk_nb<4>(dense, grid, s, parts, splits, sk, (int)total, cpr, plane, out, ldo, cols_out); break;
+    case 3: launch_splitk_nb<8>(dense, grid, s, parts, splits, sk, (int)total, cpr, plane, out, ldo, cols_out); break;
+    default: launch_splitk_nb<16>(dense, grid, s, parts, splits, sk, (int)total, cpr, plane, out, ldo, cols_out); break;
   }
   return counted_launches(1);
 }

@@ -1,8 +1,8 @@
 """The weight gradient's split-K reduction at its edges: the partial planes the
-GEMM leaves in the workspace, summed by numpy as the balanced pairwise float16
-tree over the splits (zero padded), must be dw bit for bit -- one to hundreds of
-splits, whole and partial CTAs, dense results and the patch GEMM's padded
-columns."""
+GEMM leaves in the workspace, summed by numpy as the reduction's float16 tree
+over the splits (zero padded), must be dw bit for bit -- one to hundreds of
+splits, runs of one split to 128, whole and partial CTAs, dense results and the
+patch GEMM's padded columns."""
 import numpy as np
 import pytest
 import torch
@@ -14,13 +14,21 @@ from gpu_util import dev, empty16, host, workspace
 pytestmark = pytest.mark.gpu
 
 
-def _tree(v):
+def _tree(v, chunks):
+    """The splits in aligned runs, a run summed neighbours first, the runs' sums at a
+    stride; as many runs, up to 256, as give 152 x 512 threads at one per run and chunk."""
     n = 1
     while n < v.shape[0]:
         n *= 2
     v = np.concatenate([v, np.zeros((n - v.shape[0],) + v.shape[1:], np.float16)])
-    while v.shape[0] > 1:
+    runs = 1
+    while runs < n and runs < 256 and chunks * runs < 152 * 512:
+        runs *= 2
+    while v.shape[0] > runs:
         v = v[0::2] + v[1::2]
+    while v.shape[0] > 1:
+        half = v.shape[0] // 2
+        v = v[:half] + v[half:]
     return v[0]
 
 
@@ -41,7 +49,22 @@ def test_tree_over_splits(n, h, w, c, k, r, st):
     splits = size // (2 * numel)
     assert splits > 1
     parts = ws.cpu().numpy()[:splits * numel * 2].view(np.float16).reshape(splits, numel)
-    assert np.array_equal(host(dw), _tree(parts).view(np.uint16))
+    assert np.array_equal(host(dw), _tree(parts, numel // 8).view(np.uint16))
+
+
+@pytest.mark.parametrize("n,h,c,k", [(256, 56, 256, 512), (84, 56, 1024, 1024)])
+def test_long_runs(n, h, c, k):
+    """Large results with many splits: runs of 32 and 128, which several threads share."""
+    g = torch.Generator(device="cuda").manual_seed(57)
+    f = lambda ch, std: torch.empty(n, h, h, ch, dtype=torch.float16, device="cuda").normal_(0.0, std, generator=g)
+    d = pf16.conv_desc(n, h, h, c, k, 1, 1, 1, 0)
+    size = pf16.conv_workspace_size(d, pf16.PF16_PASS_WGRAD)
+    dw, ws = empty16(k * c), workspace(size)
+    pf16.conv_wgrad(d, f(c, 1.0), f(k, 0.01), dw, ws)
+    assert pf16.sync_status() == 0
+    splits = size // (2 * k * c)
+    parts = ws.cpu().numpy()[:splits * k * c * 2].view(np.float16).reshape(splits, k * c)
+    assert np.array_equal(host(dw), _tree(parts, k * c // 8).view(np.uint16))
 
 
 def test_padded_columns():
@@ -56,4 +79,4 @@ def test_padded_columns():
     patches = n * h * h * 32 * 2  # the patch matrix comes first in the workspace (a multiple of 256 bytes)
     splits = (size - patches) // (k * 32 * 2)
     parts = ws.cpu().numpy()[patches:patches + splits * k * 64].view(np.float16).reshape(splits, k, 32)
-    assert np.array_equal(host(dw).reshape(k, 27), _tree(parts)[:, :27].view(np.uint16))
+    assert np.array_equal(host(dw).reshape(k, 27), _tree(parts, k * 4)[:, :27].view(np.uint16))
