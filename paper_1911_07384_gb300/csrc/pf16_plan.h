@@ -34,9 +34,12 @@ inline SplitkPlan splitk_plan(int splits, long long total) {
     ++p.tree_groups_log2;
   // as many groups as leave a thread at most 16 splits, and more while the GPU
   // has fewer than 512 threads per SM and a thread more than two loads (against
-  // 16 loads a thread throughout: 819 against 829 us over 24 weight gradients)
+  // 16 loads a thread throughout: 819 against 829 us over 24 weight gradients);
+  // at most 256, a CTA's threads (splits <= 4,096 keeps the first condition
+  // below that: a small result with more than 512 splits meets the second)
   p.groups_log2 = 0;
-  while (sp_log2 - p.groups_log2 > 4 || (sp_log2 - p.groups_log2 > 1 && (total << p.groups_log2) < 152ll * 512))
+  while (sp_log2 - p.groups_log2 > 4 ||
+         (p.groups_log2 < 8 && sp_log2 - p.groups_log2 > 1 && (total << p.groups_log2) < 152ll * 512))
     ++p.groups_log2;
   p.leaves_log2 = sp_log2 - p.groups_log2;
   p.leaf_step = p.groups_log2 < p.tree_groups_log2 ? 1 << p.groups_log2 : 1;

@@ -67,16 +67,28 @@ def test_long_runs(n, h, c, k):
     assert np.array_equal(host(dw), _tree(parts, k * c // 8).view(np.uint16))
 
 
-def test_padded_columns():
-    """A three-channel 3x3 convolution (patch GEMM): 27 columns of 32, the rest dropped."""
-    n, h, k = 2, 24, 64
+def _padded_columns(x, dy, n, h, k):
     d = pf16.conv_desc(n, h, h, 3, k, 3, 3, 1, 1)
-    x, dy = dev(syn.normal_f16(53, (n, h, h, 3))), dev(syn.normal_f16(54, (n, h, h, k), 0.01))
     size = pf16.conv_workspace_size(d, pf16.PF16_PASS_WGRAD)
     dw, ws = empty16(k * 27), workspace(size)
     pf16.conv_wgrad(d, x, dy, dw, ws)
     assert pf16.sync_status() == 0
     patches = n * h * h * 32 * 2  # the patch matrix comes first in the workspace (a multiple of 256 bytes)
     splits = (size - patches) // (k * 32 * 2)
-    parts = ws.cpu().numpy()[patches:patches + splits * k * 64].view(np.float16).reshape(splits, k, 32)
+    parts = ws[patches:patches + splits * k * 64].cpu().numpy().view(np.float16).reshape(splits, k, 32)
     assert np.array_equal(host(dw).reshape(k, 27), _tree(parts, k * 4)[:, :27].view(np.uint16))
+    return splits
+
+
+def test_padded_columns():
+    """A three-channel 3x3 convolution (patch GEMM): 27 columns of 32, the rest dropped."""
+    n, h, k = 2, 24, 64
+    _padded_columns(dev(syn.normal_f16(53, (n, h, h, 3))), dev(syn.normal_f16(54, (n, h, h, k), 0.01)), n, h, k)
+
+
+def test_many_splits_of_a_small_result():
+    """The same with 608 splits of 256 chunks: every thread of a CTA its own group."""
+    n, h, k = 38, 224, 64
+    g = torch.Generator(device="cuda").manual_seed(58)
+    f = lambda ch, std: torch.empty(n, h, h, ch, dtype=torch.float16, device="cuda").normal_(0.0, std, generator=g)
+    assert _padded_columns(f(3, 1.0), f(k, 0.01), n, h, k) > 512
