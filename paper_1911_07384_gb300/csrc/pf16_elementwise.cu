@@ -2004,8 +2004,9 @@ __global__ void __launch_bounds__(256)
 // rows -- contiguous in memory -- with one bulk copy into a ring, and two groups
 // of twelve warps take alternate tiles, each applying BatchNorm and ReLU in
 // place, meeting on its own barrier and scanning the windows.  So one group's
-// shared-memory pass runs under the other's window scan.  Same op sequences,
-// bit-identical results.  Batch 128 of the stem (112 x 112 x 64), statistics
+// shared-memory pass runs under the other's window scan.  Every full barrier of
+// the ring belongs to one group (ring_bars).  Same op sequences, bit-identical
+// results.  Batch 128 of the stem (112 x 112 x 64), statistics
 // closed: 91.5 -> 67.5 us (78 with one group of 30 warps, 88 with one of 16 that
 // divides for each window, 76 with three groups); 32 x 80 x 80: 18.1 -> 15.5;
 // 8 x 48 x 48: 7.7 -> 6.8.  What bounds it is the window scan's instructions: HBM
@@ -2013,6 +2014,7 @@ __global__ void __launch_bounds__(256)
 constexpr int kBpGroups = 2;
 constexpr int kBpThreads = 384;  // of a group
 constexpr int kBpStagesMax = 3;
+constexpr int kBpBarsMax = kBpStagesMax * kBpGroups;
 constexpr int kBpSmem = 220 * 1024;
 
 __global__ void __launch_bounds__(kBpGroups * kBpThreads + 32, 1)
@@ -2022,13 +2024,12 @@ __global__ void __launch_bounds__(kBpGroups * kBpThreads + 32, 1)
                         uint8_t* __restrict__ codes, uint8_t* __restrict__ mask, int N, int H, int W, int C, int P,
                         int Q, int stages, int* status, unsigned long long wait_limit_ns) {
   extern __shared__ __align__(128) uint8_t bp_smem[];
-  __shared__ uint64_t full[kBpStagesMax], empty[kBpStagesMax];
+  __shared__ uint64_t full[kBpBarsMax], empty[kBpStagesMax];
+  const int bars = ring_bars(stages, kBpGroups);  // each full barrier is one group's
   const int tc = C / 8, grp = threadIdx.x / kBpThreads, t = threadIdx.x - grp * kBpThreads;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < stages; ++s) {
-      mbar_init(smem_u32(&full[s]), 1);
-      mbar_init(smem_u32(&empty[s]), kBpThreads / 32);
-    }
+    for (int b = 0; b < bars; ++b) mbar_init(smem_u32(&full[b]), 1);
+    for (int s = 0; s < stages; ++s) mbar_init(smem_u32(&empty[s]), kBpThreads / 32);
     fence_mbar_init();
   }
   __syncthreads();
@@ -2043,34 +2044,33 @@ __global__ void __launch_bounds__(kBpGroups * kBpThreads + 32, 1)
   auto rows_of = [&](int p0) { return min(2 * kBpT + 1 - first_slot(p0), H - max(0, 2 * p0 - 1)); };
   if (grp == kBpGroups) {
     if (t == 0) {
-      int s = 0, issued = 0;
-      uint32_t ph = 0;
+      RingPos pos = ring_start(0);
+      int issued = 0;
+      uint32_t ph = 0;  // of the stages' empty barriers
       bool ok = true;
       for (int u = blockIdx.x; u < tiles; u += gridDim.x) {
         const int n = u / nb, p0 = (u - n * nb) * kBpT;
-        if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, wait_limit_ns)) {
+        if (!mbar_wait(smem_u32(&empty[pos.stage]), ph ^ 1, wait_limit_ns)) {
           ok = false;
           break;
         }
         const uint32_t bytes = (uint32_t)(rows_of(p0) * rowv) * 16u;
-        const uint32_t fb = smem_u32(&full[s]);
+        const uint32_t fb = smem_u32(&full[pos.bar]);
         mbar_arrive_expect_tx(fb, bytes);
-        bulk_load_1d(ring + s * stage_bytes + (uint32_t)(first_slot(p0) * rowv) * 16u,
+        bulk_load_1d(ring + pos.stage * stage_bytes + (uint32_t)(first_slot(p0) * rowv) * 16u,
                      reinterpret_cast<const uint4*>(x) + ((long long)n * H + max(0, 2 * p0 - 1)) * rowv, bytes, fb);
         ++issued;
-        if (++s == stages) {
-          s = 0;
-          ph ^= 1;
-        }
+        pos.advance(1, stages, bars);
+        if (pos.stage == 0) ph ^= 1;
       }
       if (!ok) {  // a consumer gave up: record it, and let the copies in flight land
         atomicExch(status, PF16_ERR_TIMEOUT);
         for (int i = 0; i < min(issued, stages); ++i) {
-          if (--s < 0) {
-            s = stages - 1;
-            ph ^= 1;
+          if (--pos.bar < 0) {
+            pos.bar = bars - 1;
+            pos.phase ^= 1;
           }
-          mbar_wait(smem_u32(&full[s]), ph, 1000000000ull);
+          mbar_wait(smem_u32(&full[pos.bar]), pos.phase, 1000000000ull);
         }
       }
     }
@@ -2086,12 +2086,11 @@ __global__ void __launch_bounds__(kBpGroups * kBpThreads + 32, 1)
   // its windows of a tile: the first one, and the step to the next
   const int tr0 = t / tc / Q, q0 = t / tc - tr0 * Q;
   const int step_r = kBpThreads / tc / Q, step_q = kBpThreads / tc - step_r * Q;
-  int s = grp;
-  uint32_t ph = 0;
+  RingPos pos = ring_start(grp);
   for (int u = blockIdx.x + grp * gridDim.x; u < tiles; u += kBpGroups * gridDim.x) {
     const int n = u / nb, p0 = (u - n * nb) * kBpT;
-    const bool got = mbar_wait(smem_u32(&full[s]), ph, wait_limit_ns);
-    uint4* zs = reinterpret_cast<uint4*>(bp_smem + s * stage_bytes);  // [2 kBpT + 1][W][tc]
+    const bool got = mbar_wait(smem_u32(&full[pos.bar]), pos.phase, wait_limit_ns);
+    uint4* zs = reinterpret_cast<uint4*>(bp_smem + pos.stage * stage_bytes);  // [2 kBpT + 1][W][tc]
     const int v0 = first_slot(p0) * rowv, v1 = got ? v0 + rows_of(p0) * rowv : 0;
     // (vectors from 2 p0's row on are this tile's to write the ReLU bits of)
     const long long mbase = ((long long)n * H + 2 * p0 - 1) * rowv;
@@ -2139,11 +2138,8 @@ __global__ void __launch_bounds__(kBpGroups * kBpThreads + 32, 1)
     }
     fence_proxy_async_smem();  // this thread's accesses, before the next copy into the stage
     __syncwarp();
-    if ((t & 31) == 0) mbar_arrive(smem_u32(&empty[s]));
-    if ((s += kBpGroups) >= stages) {
-      s -= stages;
-      ph ^= 1;
-    }
+    if ((t & 31) == 0) mbar_arrive(smem_u32(&empty[pos.stage]));
+    pos.advance(kBpGroups, stages, bars);
   }
 }
 

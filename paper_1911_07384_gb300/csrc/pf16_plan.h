@@ -2,6 +2,12 @@
 // machine that has no GPU.
 #pragma once
 
+#ifdef __CUDACC__
+#define PF16_PLAN_FN __host__ __device__ inline
+#else
+#define PF16_PLAN_FN inline
+#endif
+
 namespace pf16 {
 
 // Split-K reduction of `total` 8-column chunks over `splits` partial planes.
@@ -45,5 +51,34 @@ inline SplitkPlan splitk_plan(int splits, long long total) {
   p.leaf_step = p.groups_log2 < p.tree_groups_log2 ? 1 << p.groups_log2 : 1;
   return p;
 }
+
+// A ring of `stages` buffers that a producer fills and `groups` consumer groups
+// empty, group g taking tiles g, g + groups, ...: a position in it, one per role,
+// the producer's advanced tile by tile, a group's by `groups` (at most `stages`).
+struct RingPos {
+  int stage, bar;
+  unsigned phase;  // parity of the tile's use of its full barrier
+  PF16_PLAN_FN void advance(int by, int stages, int bars) {
+    if ((stage += by) >= stages) stage -= stages;
+    if ((bar += by) >= bars) {
+      bar -= bars;
+      phase ^= 1u;
+    }
+  }
+};
+// Full barriers.  A wait by parity is only sound for who saw the barrier's phase
+// before: until that is over, the other parity lets it pass at once.  With a
+// barrier per stage a group would meet the uses that other groups waited for
+// (three stages and two groups: every second one), and pass while the copy of
+// such a use, or its own, is in flight.  (Waiting for that use first is no way
+// out: the copy after it may already have landed, and its phase come round.)
+// With the least common multiple of both numbers each barrier serves one group,
+// which sees all of its phases.
+PF16_PLAN_FN int ring_bars(int stages, int groups) {
+  int bars = stages;
+  while (bars % groups != 0) bars += stages;
+  return bars;
+}
+PF16_PLAN_FN RingPos ring_start(int tile) { return RingPos{tile, tile, 0u}; }
 
 }  // namespace pf16

@@ -1,5 +1,6 @@
 """The launch plans of pf16_plan.h, compiled for the host on their own: the split-K
-reduction's groups of splits for every split count the weight gradients take."""
+reduction's groups of splits for every split count the weight gradients take, and the
+buffer ring of the pipelined stem pooling under every order of its events."""
 import ctypes
 import os
 import shutil
@@ -14,6 +15,12 @@ SHIM = """
 extern "C" void splitk(int splits, long long total, int* out) {
   const pf16::SplitkPlan p = pf16::splitk_plan(splits, total);
   out[0] = p.tree_groups_log2, out[1] = p.leaves_log2, out[2] = p.groups_log2, out[3] = p.leaf_step;
+}
+// stage, full barrier and parity of tiles start, start + by, ...
+extern "C" void ring(int start, int by, int stages, int groups, int n, int* out) {
+  pf16::RingPos r = pf16::ring_start(start);
+  for (int i = 0; i < n; ++i, r.advance(by, stages, pf16::ring_bars(stages, groups)))
+    out[3 * i] = r.stage, out[3 * i + 1] = r.bar, out[3 * i + 2] = (int)r.phase;
 }
 """
 
@@ -44,3 +51,51 @@ def test_splitk_groups(plans, total):
             assert step == 1
         else:
             assert leaves == 1 and groups + 1 == tree and step == 1 << groups
+
+
+def _positions(plans, start, by, stages, groups, n):
+    out = (ctypes.c_int * (3 * n))()
+    plans.ring(start, by, stages, groups, n, out)
+    return [tuple(out[3 * i:3 * i + 3]) for i in range(n)]
+
+
+@pytest.mark.parametrize("stages,groups", [(2, 2), (3, 2), (4, 2), (3, 1), (3, 3), (4, 3), (5, 3)])
+def test_ring_waits(plans, stages, groups):
+    """Every reachable order of copies issued and landed (in any order) and of groups passing
+    their waits and releasing their buffers: a wait by parity (true while the barrier's
+    present phase has the other parity) never passes before its own tile's copy has landed,
+    every tile is taken, and the schedule cannot stop."""
+    tiles = 3 * stages * groups + 2
+    prod = _positions(plans, 0, 1, stages, groups, tiles)
+    cons = {g + groups * i: p for g in range(groups)
+            for i, p in enumerate(_positions(plans, g, groups, stages, groups, (tiles - g + groups - 1) // groups))}
+    bars = 1 + max(p[1] for p in prod)
+    # state: tiles issued, those of them in flight, and each group's steps (even: waiting for
+    # its next tile, odd: holding it)
+    todo, seen = [(0, frozenset(), (0,) * groups)], set()
+    while todo:
+        state = todo.pop()
+        if state in seen:
+            continue
+        seen.add(state)
+        issued, flight, steps = state
+        landed = [u for u in range(issued) if u not in flight]
+        phase = [sum(prod[u][1] == b for u in landed) for b in range(bars)]
+        freed = [sum(prod[g + groups * i][0] == s for g in range(groups) for i in range(steps[g] // 2))
+                 for s in range(stages)]
+        nxt = [(issued, flight - {u}, steps) for u in flight]
+        if issued < tiles and freed[prod[issued][0]] == issued // stages:
+            nxt.append((issued + 1, flight | {issued}, steps))
+        for g in range(groups):
+            u = g + groups * (steps[g] // 2)
+            if u >= tiles:
+                continue
+            if steps[g] % 2 == 0:
+                stage, bar, parity = cons[u]
+                if phase[bar] % 2 == parity:
+                    continue
+                assert u in landed, f"group {g} passes the wait for tile {u} before its copy has landed: {state}"
+                assert stage == prod[u][0]
+            nxt.append((issued, flight, steps[:g] + (steps[g] + 1,) + steps[g + 1:]))
+        assert nxt or all(g + groups * (steps[g] // 2) >= tiles for g in range(groups)), f"stopped in {state}"
+        todo += nxt
