@@ -60,7 +60,28 @@ __device__ __forceinline__ uint32_t hmerge2f(uint32_t a, uint32_t b) {  // rn(a/
 }
 __device__ __forceinline__ uint32_t dup2h(uint16_t h) { return (uint32_t)h | ((uint32_t)h << 16); }
 
+// The weights na / n and nb / n of a merge with unequal counts, n = na + nb; and
+// the same out of line, for the leaf pushes of kernels with 96 registers a thread
+// (18 warps).  A push meets unequal counts only after a tensor's ragged last
+// tile, but its two divisions, inlined beside the leaf's 64 values, were more
+// than those kernels could hold: k_gemm's wide epilogue spilled 40 bytes a
+// thread, its operand transform 36, on the path of every tile.  56x56 64-256
+// forward with statistics at batch 256 98.9 -> 96.3 us, at batch 64 30.0 -> 28.3;
+// with the BatchNorm in the operand path 144.9 -> 135.9 and 41.0 -> 39.0.  (The
+// closing merges, taken once a CTA, stay inline: 96.4 and 136.2 with them out
+// of line too.  Kernels with room keep the inline form: the 3x3 64-64 forward
+// with statistics at batch 4 6.6 against 6.7 us.)
+__device__ __forceinline__ void mv2_weights(int na, int nb, uint32_t& wa, uint32_t& wb) {
+  const float n = (float)(na + nb);
+  wa = dup2h(__half_as_ushort(__float2half_rn(__fdiv_rn((float)na, n))));
+  wb = dup2h(__half_as_ushort(__float2half_rn(__fdiv_rn((float)nb, n))));
+}
+static __device__ __noinline__ void mv2_weights_call(int na, int nb, uint32_t& wa, uint32_t& wb) {
+  mv2_weights(na, nb, wa, wb);
+}
+
 // node a <- merge(a, b) with counts na, nb (the result's count is na + nb)
+template <bool TIGHT = false>
 __device__ __forceinline__ void mv2_merge(uint32_t& amu, uint32_t& av, int na, uint32_t bmu, uint32_t bv,
                                           int nb) {
   if (nb == 0) return;
@@ -75,9 +96,11 @@ __device__ __forceinline__ void mv2_merge(uint32_t& amu, uint32_t& av, int na, u
     amu = hmerge2f(amu, bmu);
     av = hadd2_rn(hmerge2f(av, bv), hmul2_rn(dh, dh));
   } else {
-    const float n = (float)(na + nb);
-    const uint32_t wa = dup2h(__half_as_ushort(__float2half_rn(__fdiv_rn((float)na, n))));
-    const uint32_t wb = dup2h(__half_as_ushort(__float2half_rn(__fdiv_rn((float)nb, n))));
+    uint32_t wa, wb;
+    if (TIGHT)
+      mv2_weights_call(na, nb, wa, wb);
+    else
+      mv2_weights(na, nb, wa, wb);
     const uint32_t wab = hmul2_rn(wa, wb);
     amu = hadd2_rn(hmul2_rn(amu, wa), hmul2_rn(bmu, wb));
     av = hadd2_rn(hadd2_rn(hmul2_rn(av, wa), hmul2_rn(bv, wb)), hmul2_rn(hmul2_rn(d, d), wab));
@@ -93,11 +116,12 @@ struct EpiStats {
 
   // leaf of chunk c from the staged tile (row r at stg + r*128, 128B-swizzled)
   // over the warp's first nv rows
+  template <bool TIGHT = false>
   __device__ __forceinline__ void leaf(int c, uint32_t stg, int lane, int nv) {
     if (nv == 32)  // a full leaf (every tile but a tensor's last): no row tests
-      leaf_impl<true, false>(c, stg, lane, 0xFFFFFFFFu, 32);
+      leaf_impl<true, false, TIGHT>(c, stg, lane, 0xFFFFFFFFu, 32);
     else
-      leaf_impl<false, false>(c, stg, lane, 0u, nv);
+      leaf_impl<false, false, TIGHT>(c, stg, lane, 0u, nv);
   }
   // the same over the rows whose bit is set in vmask (non-zero); for a prefix
   // mask this is leaf() exactly
@@ -108,7 +132,7 @@ struct EpiStats {
       leaf_impl<false, true>(c, stg, lane, vmask, __popc(vmask));
   }
   // MASK: rows tested against vmask bit by bit; else the first nv rows
-  template <bool FULL, bool MASK>
+  template <bool FULL, bool MASK, bool TIGHT = false>
   __device__ __forceinline__ void leaf_impl(int c, uint32_t stg, int lane, uint32_t vmask, int nv) {
     const uint32_t col = (uint32_t)(lane & 3) * 4;
     uint32_t x[32], t[32];  // the 32 rows' channel pair, read once
@@ -143,7 +167,7 @@ struct EpiStats {
     for (int l = 0; l < kStLevels; ++l) {
       if (cnt & (1u << l)) {
         uint32_t m2 = this->mu[c][l], v2 = this->v[c][l];
-        mv2_merge(m2, v2, n[l], mu, var, nn);
+        mv2_merge<TIGHT>(m2, v2, n[l], mu, var, nn);
         mu = m2;
         var = v2;
         nn += n[l];

@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
   static_assert(!WE || (EPI == EPI_PLAIN && !XF && BN % 128 == 0), "the wide epilogue: plain, BN 128 or 256");
   using Cfg = GemmCfg<BN, TMAE, XF, WE>;
   constexpr int CS = WE ? 2 : 1;  // column halves per tile
+  constexpr bool TIGHT = WE || XF;  // 18 warps: 96 registers a thread (mv2_weights)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -631,18 +632,24 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
       // the load modes are compile-time in each of the six pairs the plans use
       const ProducerArgs a{&mapA, &mapB, smem, full, empty, abort_flag, cid, ncl, total, lim};
       const int am = p.a_mode, bm = p.b_mode;
-      if (am == LD_TILED_K && bm == LD_TILED_K)
+      if constexpr (XF) {  // (1x1 forwards and weight gradients: two of them)
+        if (am == LD_TILED_K)
+          produce<BN, Cfg, LD_TILED_K, LD_TILED_K>(p, a);
+        else
+          produce<BN, Cfg, LD_TILED_MN, LD_TILED_MN>(p, a);
+      } else if (am == LD_TILED_K && bm == LD_TILED_K) {
         produce<BN, Cfg, LD_TILED_K, LD_TILED_K>(p, a);
-      else if (am == LD_IM2COL_K && bm == LD_TILED_K)
+      } else if (am == LD_IM2COL_K && bm == LD_TILED_K) {
         produce<BN, Cfg, LD_IM2COL_K, LD_TILED_K>(p, a);
-      else if (am == LD_TILED_K && bm == LD_TILED_MN)
+      } else if (am == LD_TILED_K && bm == LD_TILED_MN) {
         produce<BN, Cfg, LD_TILED_K, LD_TILED_MN>(p, a);
-      else if (am == LD_IM2COL_K && bm == LD_TAP3D_MN)
+      } else if (am == LD_IM2COL_K && bm == LD_TAP3D_MN) {
         produce<BN, Cfg, LD_IM2COL_K, LD_TAP3D_MN>(p, a);
-      else if (am == LD_TILED_MN && bm == LD_TILED_MN)
+      } else if (am == LD_TILED_MN && bm == LD_TILED_MN) {
         produce<BN, Cfg, LD_TILED_MN, LD_TILED_MN>(p, a);
-      else
+      } else {
         produce<BN, Cfg, LD_TILED_MN, LD_IM2COL_MN>(p, a);
+      }
     }
   } else if (warp == 1) {
     if (elect_one()) {
@@ -838,7 +845,7 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
               stats.leaf_bwd(c / 64, stg, lane, nv, bin);
               if (c + 64 < BN && n0 + c + 64 < p.N) bin.load(p, (long long)(m0 + sub * 32), n0 + c + 64, nv, lane);
             } else {
-              stats.leaf(c / 64, stg, lane, nv);
+              stats.leaf<TIGHT>(c / 64, stg, lane, nv);
             }
           }
         }
