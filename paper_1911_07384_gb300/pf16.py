@@ -82,9 +82,6 @@ class BnTensors(ctypes.Structure):
     _fields_ = [(n, ctypes.c_void_p) for n in _BN_T]
 
 
-_BN_FIELDS = frozenset(_BN_T)
-
-
 _lock = threading.Lock()
 _lib = None
 
@@ -316,9 +313,7 @@ def bn_workspace_size(d: BnDesc) -> int:
 
 def _bn_tensors(tensors):
     t = BnTensors()
-    for k, v in tensors.items():
-        if k not in _BN_FIELDS:
-            raise TypeError(f"unexpected BatchNorm tensor {k!r}")
+    for k, v in tensors.items():  # (a name that is no field is ignored, as the constructor does)
         if v is not None:
             setattr(t, k, v.data_ptr())
     return t
