@@ -190,8 +190,11 @@ def _stream(stream):
             import torch
 
             torch.cuda.init()
-            get, dev = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-            _raw_stream = lambda: get(dev())
+            get, dev = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+            if get and dev:
+                _raw_stream = lambda: get(dev())
+            else:  # (a torch without these two, which are not public)
+                _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
         return _raw_stream()
     if isinstance(stream, int):
         return stream
