@@ -681,7 +681,7 @@ def time_bn(shape, bn_pass, steps, warmup):
 KERNEL_LAYER = (256, 56, 56, 64, 256, 1, 1, 1, 0)
 KERNEL_NAME = "k_gemm<256> (plain epilogue, forward statistics), 56x56 64->256 1x1 forward, batch 256"
 TRAFFIC_JSON = os.path.join(ROOT, "profiles", "k_gemm_256_conv_56x56_64to256_fwd_stats_b256_traffic.json")
-GEMM_SOURCES = ["pf16_gemm.cu", "pf16_epi.cuh", "pf16_api.cu", "pf16_internal.h", "pf16_ptx.cuh"]
+GEMM_SOURCES = ["pf16_gemm.cu", "pf16_epi.cuh", "pf16_api.cu", "pf16_internal.h", "pf16_plan.h", "pf16_ptx.cuh"]
 
 
 def wgrad_is_gemm(h, w, c, k, r, s, st, pad):

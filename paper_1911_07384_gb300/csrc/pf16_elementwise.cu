@@ -11,7 +11,6 @@
 
 #include "../../include/pf16.h"
 #include "pf16_internal.h"
-#include "pf16_plan.h"
 #include "pf16_ptx.cuh"
 
 namespace pf16 {

@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(XF ? kGemmThreadsXf : (WE ? kGemmThreadsWide :
 
   if (warp == 0) {
     if (elect_one()) {
-      // the load modes are compile-time in each of the six pairs the plans use
+      // the load modes are compile-time in each of the six pairs that gemm_modes_ok lets through
       const ProducerArgs a{&mapA, &mapB, smem, full, empty, abort_flag, cid, ncl, total, lim};
       const int am = p.a_mode, bm = p.b_mode;
       if constexpr (XF) {  // (1x1 forwards and weight gradients: two of them)
@@ -1010,6 +1010,7 @@ static cudaError_t launch_bn_t(const CUtensorMap& mA, const CUtensorMap& mB, con
 cudaError_t launch_gemm(int BN, const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mC,
                         const GemmParams& p, int grid, cudaStream_t s, const CUtensorMap* mX,
                         const CUtensorMap* mD) {
+  if (!gemm_modes_ok(p.a_mode, p.b_mode, p.xf_operand != 0)) return cudaErrorInvalidValue;
   // the BatchNorm-input and addend maps (unused without backward statistics)
   const CUtensorMap& x = mX ? *mX : mC;
   const CUtensorMap& d = mD ? *mD : x;

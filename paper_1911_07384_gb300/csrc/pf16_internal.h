@@ -6,6 +6,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "pf16_plan.h"
+
 namespace pf16 {
 
 // Kernels this library has enqueued in the process (launches recorded into a
@@ -59,13 +61,7 @@ inline cudaError_t counted_launches(int n) {
 //                 64(k) x 64(c) slice of one tap, MN-major B of the data
 //                 gradient (no transposed weight copy is needed).
 // ---------------------------------------------------------------------------
-enum LoadMode : int {
-  LD_TILED_K = 0,
-  LD_TILED_MN = 1,
-  LD_IM2COL_K = 2,
-  LD_IM2COL_MN = 3,
-  LD_TAP3D_MN = 4
-};
+// (enum LoadMode: pf16_plan.h, with the pairs that the kernel is compiled for)
 enum OutMode : int { OUT_STORE = 0, OUT_ACCUM = 1, OUT_PARTIAL = 2 };
 
 constexpr int kMaxTaps = 49;

@@ -10,6 +10,24 @@
 
 namespace pf16 {
 
+enum LoadMode : int {
+  LD_TILED_K = 0,
+  LD_TILED_MN = 1,
+  LD_IM2COL_K = 2,
+  LD_IM2COL_MN = 3,
+  LD_TAP3D_MN = 4
+};
+
+// Whether k_gemm's producer is compiled for A in mode a and B in mode b: forward
+// (1x1, others), data gradient (1x1, stride phases), weight gradient (1x1 and
+// patches, others); with an operand transform only the 1x1 forward and weight
+// gradient.  Any other pair is refused before a launch.
+inline bool gemm_modes_ok(int a, int b, bool transform) {
+  if (a == LD_TILED_K) return b == LD_TILED_K || (b == LD_TILED_MN && !transform);
+  if (a == LD_TILED_MN) return b == LD_TILED_MN || (b == LD_IM2COL_MN && !transform);
+  return a == LD_IM2COL_K && (b == LD_TILED_K || b == LD_TAP3D_MN) && !transform;
+}
+
 // Split-K reduction of `total` 8-column chunks over `splits` partial planes.
 //
 // The tree over the splits, padded with zeros to a power of two, is part of the

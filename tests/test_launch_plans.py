@@ -1,6 +1,7 @@
 """The launch plans of pf16_plan.h, compiled for the host on their own: the split-K
-reduction's groups of splits for every split count the weight gradients take, and the
-buffer ring of the pipelined stem pooling under every order of its events."""
+reduction's groups of splits for every split count the weight gradients take, the
+buffer ring of the pipelined stem pooling under every order of its events, and the load
+modes that the GEMM is launched with."""
 import ctypes
 import os
 import shutil
@@ -16,6 +17,7 @@ extern "C" void splitk(int splits, long long total, int* out) {
   const pf16::SplitkPlan p = pf16::splitk_plan(splits, total);
   out[0] = p.tree_groups_log2, out[1] = p.leaves_log2, out[2] = p.groups_log2, out[3] = p.leaf_step;
 }
+extern "C" int modes_ok(int a, int b, int transform) { return pf16::gemm_modes_ok(a, b, transform != 0); }
 // stage, full barrier and parity of tiles start, start + by, ...
 extern "C" void ring(int start, int by, int stages, int groups, int n, int* out) {
   pf16::RingPos r = pf16::ring_start(start);
@@ -99,3 +101,14 @@ def test_ring_waits(plans, stages, groups):
             nxt.append((issued, flight, steps[:g] + (steps[g] + 1,) + steps[g + 1:]))
         assert nxt or all(g + groups * (steps[g] // 2) >= tiles for g in range(groups)), f"stopped in {state}"
         todo += nxt
+
+
+def test_gemm_load_modes(plans):
+    """Six pairs, two of them with an operand transform; every other is refused."""
+    tiled_k, tiled_mn, im2col_k, im2col_mn, tap3d_mn = range(5)
+    pairs = {(tiled_k, tiled_k), (im2col_k, tiled_k), (tiled_k, tiled_mn), (im2col_k, tap3d_mn),
+             (tiled_mn, tiled_mn), (tiled_mn, im2col_mn)}
+    for a in range(-1, 7):
+        for b in range(-1, 7):
+            assert bool(plans.modes_ok(a, b, 0)) == ((a, b) in pairs)
+            assert bool(plans.modes_ok(a, b, 1)) == ((a, b) in {(tiled_k, tiled_k), (tiled_mn, tiled_mn)})
