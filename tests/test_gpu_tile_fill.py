@@ -21,7 +21,6 @@ CASES = [(14, 14, 128, 256, 1, 1, 3, 80), (14, 14, 64, 320, 3, 1, 2, 60), (16, 1
 
 @pytest.mark.parametrize("h,w,c,k,r,st,small,large", CASES)
 def test_tile_width(h, w, c, k, r, st, small, large):
-    x = torch.from_numpy(syn.normal_f16(41, (1, h, w, c)).view(np.int16)).cuda()
     g = torch.Generator(device="cuda").manual_seed(5)
     p, q = (h + 2 * (r // 2) - r) // st + 1, (w + 2 * (r // 2) - r) // st + 1
     f = lambda *s: torch.randn(s, device="cuda", generator=g).to(torch.float16)
