@@ -2186,89 +2186,100 @@ cudaError_t launch_bn_relu_pool_fwd(const BnLaunch& b, const uint8_t* conv_stats
 // Global average pooling (halving tree over hw padded to 2^L, x rn(2^L/hw)).
 // Bound by HBM: x is read once forward, written once backward.
 //
-// Forward: a CTA takes 32 channel groups of 8 (a warp reads 512 consecutive
-// bytes of a pixel); its warps share the padded pixels in aligned runs of
-// 2^L / 8 (at least 8), each summed as perfect subtrees of 8 with all eight
-// loads in flight, and the runs' nodes meet in shared memory -- the same
+// Forward: a warp reads 32 channel groups of 8 (512 consecutive bytes) of a
+// pixel; up to eight warps share the padded pixels of the same groups in aligned
+// runs of 2^L / 8 (at least 8), each summed as perfect subtrees of 8 with all
+// eight loads in flight, and the runs' nodes meet in shared memory -- the same
 // perfect tree as a pixel-by-pixel counter, whose one load in flight per
-// thread made 256 x 49 x 2048 take 37.5 us (1.4 TB/s); now 17 us.
+// thread made 256 x 49 x 2048 take 37.5 us (1.4 TB/s); now 17 us.  With fewer
+// than 64 padded pixels a CTA's eight warps take several sets of groups (one set
+// a CTA left warps idle: 256 x 1 x 2048 4.6 -> 1.7 us, 256 x 9 x 2048 5.6 -> 3.1).
 // Backward: a thread scales its channel group once and writes it to every
-// eighth pixel (15.3 -> 12.2 us at that size).
+// eighth pixel (15.3 -> 12.2 us at that size); with four pixels or fewer a CTA
+// likewise takes several sets (256 x 1 x 2048 2.2 -> 1.4 us).
 // ============================================================================
 constexpr int kPoolWarps = 8;
+constexpr int kPoolWarpsLog2 = 3;
 
+// 2^warps_log2 warps per 32 channel groups
 __global__ void __launch_bounds__(32 * kPoolWarps)
     k_avgpool_fwd(const uint16_t* __restrict__ x, uint16_t* __restrict__ y, int N, int HW, int C, int levels,
-                  uint16_t ratio) {
+                  int warps_log2, uint16_t ratio) {
   pdl_wait();
   __shared__ uint4 node[kPoolWarps][32];
   const int tc = C / 8, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int warps = 1 << warps_log2, part = w & (warps - 1);
   const long long total = (long long)N * tc;
-  const long long t = (long long)blockIdx.x * 32 + lane;
-  // warps in use and pixels per warp (powers of two; run * warps = 2^levels)
-  const int warps = levels <= 3 ? 1 : (levels >= 6 ? kPoolWarps : 1 << (levels - 3));
-  const int run = (1 << levels) / warps;
-  const int nb = run < 8 ? run : 8;  // leaves per batch
-  if (w < warps) {
-    const int cg = t < total ? (int)(t % tc) : 0;
-    const long long n = t < total ? t / tc : 0;
-    const uint4* src = reinterpret_cast<const uint4*>(x) + n * HW * tc + cg;
-    uint4 acc = zero4();
-    Tree4<12, true> tree;  // over the run's batches, when it has several
-    for (int i0 = 0; i0 < run; i0 += 8) {
-      uint4 v[8];
+  const long long set = ((long long)blockIdx.x << (kPoolWarpsLog2 - warps_log2)) + (w >> warps_log2);
+  const long long t = set * 32 + lane;
+  const int run = 1 << (levels - warps_log2);  // pixels per warp
+  const int nb = run < 8 ? run : 8;            // leaves per batch
+  const int cg = t < total ? (int)(t % tc) : 0;
+  const long long n = t < total ? t / tc : 0;
+  const uint4* src = reinterpret_cast<const uint4*>(x) + n * HW * tc + cg;
+  uint4 acc = zero4();
+  Tree4<12, true> tree;  // over the run's batches, when it has several
+  for (int i0 = 0; i0 < run; i0 += 8) {
+    uint4 v[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int px = w * run + i0 + i;
-        v[i] = (t < total && i < nb && px < HW) ? __ldg(src + (long long)px * tc) : zero4();
-      }
-#pragma unroll
-      for (int h = 1; h < 8; h *= 2)
-#pragma unroll
-        for (int i = 0; i < 8; i += 2 * h)
-          if (i + h < nb) v[i] = hmerge4(v[i], v[i + h]);
-      if (run <= 8) {
-        acc = v[0];
-        break;
-      }
-      tree.push(v[0]);
+    for (int i = 0; i < 8; ++i) {
+      const int px = part * run + i0 + i;
+      v[i] = (t < total && i < nb && px < HW) ? __ldg(src + (long long)px * tc) : zero4();
     }
-    if (run > 8) acc = tree.finish(ceil_log2(run / 8));
-    node[w][lane] = acc;
+#pragma unroll
+    for (int h = 1; h < 8; h *= 2)
+#pragma unroll
+      for (int i = 0; i < 8; i += 2 * h)
+        if (i + h < nb) v[i] = hmerge4(v[i], v[i + h]);
+    if (run <= 8) {
+      acc = v[0];
+      break;
+    }
+    tree.push(v[0]);
   }
-  __syncthreads();
-  if (w != 0 || t >= total) return;
-  uint4 v[kPoolWarps];
+  if (run > 8) acc = tree.finish(ceil_log2(run / 8));
+  if (warps > 1) {
+    node[w][lane] = acc;
+    __syncthreads();
+    if (part != 0) return;
+    uint4 v[kPoolWarps];
 #pragma unroll
-  for (int i = 0; i < kPoolWarps; ++i) v[i] = i < warps ? node[i][lane] : zero4();
+    for (int i = 0; i < kPoolWarps; ++i) v[i] = i < warps ? node[w + i][lane] : zero4();
 #pragma unroll
-  for (int h = 1; h < kPoolWarps; h *= 2)
+    for (int h = 1; h < kPoolWarps; h *= 2)
 #pragma unroll
-    for (int i = 0; i < kPoolWarps; i += 2 * h)
-      if (i + h < warps) v[i] = hmerge4(v[i], v[i + h]);
-  reinterpret_cast<uint4*>(y)[t] = mul4(v[0], dup2(ratio));
+      for (int i = 0; i < kPoolWarps; i += 2 * h)
+        if (i + h < warps) v[i] = hmerge4(v[i], v[i + h]);
+    acc = v[0];
+  }
+  if (t < total) reinterpret_cast<uint4*>(y)[t] = mul4(acc, dup2(ratio));
 }
 
 __global__ void __launch_bounds__(32 * kPoolWarps)
-    k_avgpool_bwd(const uint16_t* __restrict__ dy, uint16_t* __restrict__ dx, int N, int HW, int C, uint16_t inv) {
+    k_avgpool_bwd(const uint16_t* __restrict__ dy, uint16_t* __restrict__ dx, int N, int HW, int C, int warps_log2,
+                  uint16_t inv) {
   pdl_wait();
   const int tc = C / 8, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long t = (long long)blockIdx.x * 32 + lane;
+  const int warps = 1 << warps_log2, part = w & (warps - 1);
+  const long long set = ((long long)blockIdx.x << (kPoolWarpsLog2 - warps_log2)) + (w >> warps_log2);
+  const long long t = set * 32 + lane;
   if (t >= (long long)N * tc) return;
   const long long n = t / tc;
   const int cg = (int)(t - n * tc);
   const uint4 v = mul4(__ldg(reinterpret_cast<const uint4*>(dy) + t), dup2(inv));
   uint4* dst = reinterpret_cast<uint4*>(dx) + n * HW * tc + cg;
-  for (long long px = blockIdx.y * kPoolWarps + w; px < HW; px += gridDim.y * kPoolWarps) dst[px * tc] = v;
+  for (long long px = blockIdx.y * warps + part; px < HW; px += gridDim.y * warps) dst[px * tc] = v;
 }
 
 cudaError_t launch_avgpool_fwd(const uint16_t* x, uint16_t* y, int N, int HW, int C,
                                cudaStream_t s) {
-  int L = 0;
-  while ((1 << L) < HW) ++L;
+  const int L = ceil_log2(HW);
   const uint16_t ratio = f16_bits_host((float)((double)(1 << L) / HW));
   const long long total = (long long)N * (C / 8);
-  launch_pdl(k_avgpool_fwd, dim3((unsigned)((total + 31) / 32)), dim3(32 * kPoolWarps), 0, s, x, y, N, HW, C, L, ratio);
+  const int warps_log2 = std::min(std::max(L - 3, 0), kPoolWarpsLog2);
+  const long long per_cta = 32ll << (kPoolWarpsLog2 - warps_log2);  // channel groups
+  launch_pdl(k_avgpool_fwd, dim3((unsigned)((total + per_cta - 1) / per_cta)), dim3(32 * kPoolWarps), 0, s, x, y, N,
+             HW, C, L, warps_log2, ratio);
   return counted_launches(1);
 }
 
@@ -2276,11 +2287,14 @@ cudaError_t launch_avgpool_bwd(const uint16_t* dy, uint16_t* dx, int N, int HW, 
                                cudaStream_t s) {
   const uint16_t inv = f16_bits_host((float)(1.0 / HW));
   const long long total = (long long)N * (C / 8);
+  const int warps_log2 = std::min(ceil_log2(HW), kPoolWarpsLog2);
+  const long long per_cta = 32ll << (kPoolWarpsLog2 - warps_log2);
   // the pixels of an image are shared by gridDim.y CTAs where the channel groups
   // alone leave SMs idle (16 CTAs per SM wanted)
-  const long long gx = (total + 31) / 32;
+  const long long gx = (total + per_cta - 1) / per_cta;
   const long long gy = std::max(1ll, std::min((HW + kPoolWarps - 1ll) / kPoolWarps, kGb300Sms * 16 / gx));
-  launch_pdl(k_avgpool_bwd, dim3((unsigned)gx, (unsigned)gy), dim3(32 * kPoolWarps), 0, s, dy, dx, N, HW, C, inv);
+  launch_pdl(k_avgpool_bwd, dim3((unsigned)gx, (unsigned)gy), dim3(32 * kPoolWarps), 0, s, dy, dx, N, HW, C,
+             warps_log2, inv);
   return counted_launches(1);
 }
 

@@ -1,6 +1,7 @@
 """The head's kernels at the edges of their splits, bit for bit: the average
 pooling's halving tree over padded pixels (runs of one, several and many
-batches per warp), and the loss's column and loss trees over row segments.
+batches per warp; one to eight sets of channel groups per CTA), and the loss's
+column and loss trees over row segments.
 The expected trees are numpy float16 arithmetic (correctly rounded adds;
 a/2 + rn(b/2) formed exactly in binary64 and rounded once)."""
 import numpy as np
@@ -34,7 +35,7 @@ def _f16(bits):
 
 
 @pytest.mark.parametrize("N,HW,C", [(3, 1, 8), (2, 2, 264), (5, 7, 64), (1, 8, 8), (2, 9, 40), (3, 33, 72), (2, 65, 8),
-                                    (1, 2049, 8)])
+                                    (1, 2049, 8), (70, 3, 72), (50, 12, 40), (40, 20, 72), (300, 1, 8)])
 def test_avgpool_tree(N, HW, C):
     x = syn.normal_f16(31, (N, HW, C))
     y, dx = empty16(N * C), empty16(N * HW * C)
