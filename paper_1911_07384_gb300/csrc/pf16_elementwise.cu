@@ -2062,15 +2062,14 @@ __global__ void __launch_bounds__(kBpGroups * kBpThreads + 32, 1)
         pos.advance(1, stages, bars);
         if (pos.stage == 0) ph ^= 1;
       }
-      if (!ok) {  // a consumer gave up: record it, and let the copies in flight land
-        atomicExch(status, PF16_ERR_TIMEOUT);
-        for (int i = 0; i < min(issued, stages); ++i) {
-          if (--pos.bar < 0) {
-            pos.bar = bars - 1;
-            pos.phase ^= 1;
-          }
-          mbar_wait(smem_u32(&full[pos.bar]), pos.phase, 1000000000ull);
+      if (!ok) atomicExch(status, PF16_ERR_TIMEOUT);  // a consumer gave up
+      // the last copies have landed when the CTA ends, also where the consumers left without them
+      for (int i = 0; i < min(issued, stages); ++i) {
+        if (--pos.bar < 0) {
+          pos.bar = bars - 1;
+          pos.phase ^= 1;
         }
+        mbar_wait(smem_u32(&full[pos.bar]), pos.phase, 1000000000ull);
       }
     }
     return;
