@@ -2005,8 +2005,8 @@ __global__ void __launch_bounds__(256)
 // place, meeting on its own barrier and scanning the windows.  So one group's
 // shared-memory pass runs under the other's window scan.  Every full barrier of
 // the ring belongs to one group (ring_bars).  Same op sequences, bit-identical
-// results.  Batch 128 of the stem (112 x 112 x 64), statistics
-// closed: 91.5 -> 67.5 us (78 with one group of 30 warps, 88 with one of 16 that
+// results.  Batch 128 of the stem (112 x 112 x 64), statistics closed: 91.5 ->
+// 67.5 us, 63.6 since (78 with one group of 30 warps, 88 with one of 16 that
 // divides for each window, 76 with three groups); 32 x 80 x 80: 18.1 -> 15.5;
 // 8 x 48 x 48: 7.7 -> 6.8.  What bounds it is the window scan's instructions: HBM
 // would take 44 us at batch 128.

@@ -1153,11 +1153,11 @@ __device__ __forceinline__ void halo3_combine(uint32_t tb, int lane, bool f32, b
 // so that a drain never waits for the previous tile's store, and the statistics
 // taken from them by eight more warps.  In one chain, drain and statistics of a
 // tile took ~2,400 cycles of its epilogue group, above twice the ~1,000 cycles
-// of its MMAs.  Batch 128 of the 224 x 224 stem, with the space-to-depth pass's
-// 19 us: with statistics 93.0 -> 82.3 us, without 81.2 -> 71.8; 32 x 160 x 160
-// with statistics 22.5 -> 21.0.  Statistics warp e takes epilogue warp e's tiles
-// in their order, so the trees are the same.  What bounds it now is the MMAs
-// (~62 cycles each at N = 64) and the output's stores, ~50 us each.
+// of its MMAs.  Batch 128 of the 224 x 224 stem, the space-to-depth pass
+// included: with statistics 91.2 -> 81.3 us, without 79.5 -> 69.9; 32 x 160 x
+// 160 with statistics 22.4 -> 21.0.  Statistics warp e takes epilogue warp e's
+// tiles in their order, so the trees are the same.  What bounds it now is the
+// MMAs (~62 cycles each at N = 64) and the output's stores, ~50 us each.
 template <int CB, bool BS, bool SW>
 __global__ void __launch_bounds__(SW ? kHaloThreadsSw : kGemmThreads, 1)
     k_gemm_halo(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,

@@ -272,7 +272,7 @@ cudaError_t launch_sgd(uint16_t* w, uint16_t* v, const uint16_t* g, size_t n, ui
 cudaError_t launch_wait_flag(const uint32_t* flag, uint32_t value, unsigned long long limit_ns, int* status,
                              cudaStream_t s);
 // sum of `splits` FP16 partial matrices [splits][rows][cols] by a balanced
-// pairwise tree; the result row r goes to out + r*ldo (only cols_out columns).
+// pairwise tree (pf16_plan.h); the result row r goes to out + r*ldo (only cols_out columns).
 // Data-parallel exchange, combining step (pf16_allreduce_combine): n and
 // plane_stride multiples of 8, 1 <= world <= 1024.
 cudaError_t launch_dp_combine(const uint16_t* planes, int world, size_t n, size_t plane_stride, uint16_t scale,
